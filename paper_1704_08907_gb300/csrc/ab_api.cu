@@ -216,6 +216,22 @@ ab_status ensure_scan(ab_ctx* c, int64_t items) {
     return AB_OK;
 }
 
+// Workspace of the FP32 dense walks' partial sums, or NULL, on which they run
+// unsplit (slower on few rows, never refused): when the memory is not to be
+// had, and under stream capture, where a captured call would keep a pointer
+// that a later, larger call frees.
+void* dense_scratch(ab_ctx* c, size_t need) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (need == 0) return nullptr;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (cap != cudaStreamCaptureStatusNone) return nullptr;
+    return grow(&c->sc.dense_ws, &c->sc.cap_dense_ws, need, c->stream) == cudaSuccess ? c->sc.dense_ws
+                                                                                     : nullptr;
+}
+
 ab_status require_cells(ab_ctx* c) {
     if (!c->cl.valid)
         return fail(c, AB_ERR_STALE, "no current cell list: call ab_build after creating the "
@@ -684,7 +700,8 @@ ab_status ab_kernel_matvec(ab_ctx* c, int64_t m, int64_t n, const float* X, cons
     if (!dg.ok) return fail(c, AB_ERR_CUDA, "cannot make device %d current", c->device);
     cudaError_t e;
     if (prec == AB_PREC_FP32) {
-        e = ab::launch_dense_fwd(m, n, (const float4*)X, (const float4*)Y, nrhs, W, s, prec, out,
+        void* ws = dense_scratch(c, ab::dense_fwd_workspace_bytes(m, n, nrhs));
+        e = ab::launch_dense_fwd(m, n, (const float4*)X, (const float4*)Y, nrhs, W, s, out, ws,
                                  c->stream);
     } else {
         if (nrhs != 64)
@@ -721,14 +738,19 @@ ab_status ab_kernel_solve(ab_ctx* c, int64_t n, const float* X, int32_t nrhs, co
     if (!dg.ok) return fail(c, AB_ERR_CUDA, "cannot make device %d current", c->device);
     cudaError_t e = grow(&c->sc.solve_ws, &c->sc.cap_solve_ws, ab::solve_workspace_bytes(n, nrhs),
                          c->stream);
-    if (e == cudaSuccess && prec != AB_PREC_FP32)
+    void* ws = nullptr;
+    if (prec == AB_PREC_FP32) {
+        ws = dense_scratch(c, ab::dense_fwd_workspace_bytes(n, n, nrhs));
+    } else if (e == cudaSuccess) {
         e = grow(&c->sc.dense_ws, &c->sc.cap_dense_ws, ab::dense_tc_workspace_bytes(n), c->stream);
+        ws = c->sc.dense_ws;
+    }
     if (e != cudaSuccess) return cuda_fail(c, e, "ab_kernel_solve workspace");
     const float4* X4 = (const float4*)X;
     const ab::SolveMatvec mv = [&](const float* P, float* Q) -> cudaError_t {
-        if (prec == AB_PREC_FP32) return ab::launch_dense_fwd(n, n, X4, X4, nrhs, P, s, prec, Q, c->stream);
-        return ab::launch_dense_tc_fwd(n, n, X4, X4, nrhs, P, s, prec, Q, c->sc.dense_ws, c->d_err,
-                                       c->stream);
+        if (prec == AB_PREC_FP32)
+            return ab::launch_dense_fwd(n, n, X4, X4, nrhs, P, s, Q, ws, c->stream);
+        return ab::launch_dense_tc_fwd(n, n, X4, X4, nrhs, P, s, prec, Q, ws, c->d_err, c->stream);
     };
     int it = 0;
     float rr = 0.0f;
@@ -766,15 +788,20 @@ ab_status ab_kernel_matvec_bwd(ab_ctx* c, int64_t m, int64_t n, const float* X, 
     if (!dg.ok) return fail(c, AB_ERR_CUDA, "cannot make device %d current", c->device);
     double* partial = nullptr;
     if (ds) {
-        // SIMT: one partial per 128-row block; tensor cores: up to two per block
-        if ((st = ensure_partial(c, 2 * (size_t)ab::dense_partial_capacity(m, n) + 2)) != AB_OK) return st;
+        // FP32: one partial per block; tensor cores: up to two per 128-row block
+        const size_t count = prec == AB_PREC_FP32 ? ab::dense_partial_capacity(m, n, nrhs)
+                                                  : 2 * ((size_t)(m + 127) / 128) + 2;
+        if ((st = ensure_partial(c, count)) != AB_OK) return st;
         partial = c->sc.partial;
     }
     int pc = 0;
     cudaError_t e;
     if (prec == AB_PREC_FP32) {
-        e = ab::launch_dense_bwd(m, n, (const float4*)X, (const float4*)Y, nrhs, W, s, prec, G, dW,
-                                 (float4*)dX, (float4*)dY, partial, &pc, c->stream);
+        void* ws = dense_scratch(c, ab::dense_bwd_workspace_bytes(
+                                        m, n, nrhs, dW != nullptr, dX != nullptr, dY != nullptr,
+                                        ds != nullptr));
+        e = ab::launch_dense_bwd(m, n, (const float4*)X, (const float4*)Y, nrhs, W, s, G, dW,
+                                 (float4*)dX, (float4*)dY, partial, &pc, ws, c->stream);
     } else {
         if (nrhs != 64)
             return fail(c, AB_ERR_UNSUPPORTED, "tensor-core paths need nrhs == 64");

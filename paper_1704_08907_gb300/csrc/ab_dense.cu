@@ -2,18 +2,38 @@
 // and its adjoint (the RBF / Gaussian-process operators of paper Sec. 1 and
 // Sec. 1.1; dense global operators, Sec. 2.2.2) on FP32 CUDA cores.
 //
-// Forward (k_dense_fwd): a CTA owns 128 rows of X and all (<= 64) columns of
-// W.  For each chunk of 32 Y points it stages Y and W in shared memory,
-// evaluates the 128 x 32 kernel tile once (direct differences, FP32, exp via
-// ex2), and then runs a 128 x 64 x 32 register-tiled product with each
-// thread holding an 8 x 4 accumulator tile in packed FP32 pairs.  The exponentials are 1/64 of the
-// multiply-adds, so the kernel is bound by the FP32 pipe.
+// One kernel, k_dense_own, serves the forward and every gradient.  Each
+// thread owns I points (its rows) and walks a range of the other points,
+// staged in shared memory and read as broadcasts; per pair it evaluates
+// d = o - y, |d|^2 and K = 2^(-s log2e |d|^2) once and adds to
+//   VAL   v_o[c] += K B[c]             (the product, or dW with roles swapped)
+//   GRAD  S = sum_c A_o[c] B[c],  g_o += S K d,  e_o += S K |d|^2
+//         (dX and ds, or dY with roles swapped)
+// in registers.  VAL and GRAD together give dW and dY in one walk.
 //
-// Adjoint: dW = K^T G is the forward with the roles of (X, W) and (Y, G)
-// swapped (K(X,Y)^T = K(Y,X)); dX (and ds) come from k_dense_gradx, which for
-// each 128-row block forms S = G W_chunk^T on CUDA cores, A = S o K, and the
-// row reductions sum_j A_ij, sum_j A_ij y_j, sum_j A_ij d_ij^2; dY is the same
-// kernel with (X, G) and (Y, W) swapped.
+// Why this shape (65,536^2 pairs unless a size is given; the form before it
+// was a 128 x 64 tile product through shared memory, always 64 columns wide,
+// one block per 128 rows, and a separate scalar gradient kernel):
+//  - The right-hand sides are compiled in powers of two (R), so one target
+//    costs 8 FP32 operations a pair and not 7 + 64.
+//  - Distances are formed for two rows at once and products for two columns
+//    at once (f32x2: half the issue slots; the FP32 pipe itself runs 128
+//    lane-operations a clock per SM either way).
+//  - A broadcast shared load of 16 bytes takes about two clocks of the SM's
+//    shared-memory pipe, so it has to feed many operations: I = 4 rows a
+//    thread (2 where the gradient's registers leave no room).
+//  - Few rows leave the chip idle, so the walk is split over the other
+//    points as well (plan_split); the splits' partial sums are combined in a
+//    fixed order by k_dense_combine, so results do not depend on timing.
+//
+// Bound: the FP32 pipe (7 + R operations a pair for values, 12 + R for
+// gradients, 128 a clock per SM).  Measured against the tile form, forward /
+// whole adjoint, us (and the forward's time at the pipe's rate):
+//   65,536 x 65,536, 64 columns   16,129 / 67,786 -> 12,213 / 35,809  (8,038)
+//   65,536 x 65,536,  1 column    16,042 / 66,625 ->  1,018 /  3,516    (906)
+//   16,384 x 16,384, 32 columns    1,465 /  5,851 ->    445 /  1,263    (276)
+//    5,001 x 12,345, 16 columns    1,102 /  2,783 ->     80 /    211     (37)
+//    2,000 x 30,000,  1 column     2,649 /  4,479 ->     32 /     87     (13)
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -23,10 +43,7 @@ namespace ab {
 
 namespace {
 
-constexpr int kBM = 128;      // X rows per CTA
-constexpr int kBN = 32;       // Y points per chunk
-constexpr int kRHS = 64;      // padded right-hand-side width
-constexpr int kDThreads = 256;
+constexpr int kOwnThreads = 128;
 constexpr float kLog2eD = 1.4426950408889634f;
 
 __device__ __forceinline__ float ex2f(float x) {
@@ -35,7 +52,7 @@ __device__ __forceinline__ float ex2f(float x) {
     return y;
 }
 
-// Packed FP32 pairs: fma.rn.f32x2 rounds each half exactly like fmaf.
+// Packed FP32 pairs: each half rounds exactly like the scalar operation.
 __device__ __forceinline__ uint64_t f2p(float a, float b) {
     uint64_t r;
     asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
@@ -49,225 +66,479 @@ __device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
+__device__ __forceinline__ uint64_t fmul2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t fsub2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 
-// thread layout for the product: tx in [0,16) -> 4 columns, ty in [0,16) ->
-// 8 consecutive rows ty*8 .. ty*8+7 (two float4 shared loads; a warp's two ty
-// values read broadcast addresses).  Rows are paired in fma.f32x2 (the K
-// values of rows 2r, 2r+1 sit in an aligned register pair of the float4 load;
-// the W value is duplicated), 16 packed FMAs a K step instead of 32, with
-// the same rounding and order as scalar FMAs (65,536^2 x 64: 17.4 -> 16.0
-// ms, outputs bit-identical).  W and Y chunks alternate between two shared
-// buffers.
-__global__ void __launch_bounds__(kDThreads)
-k_dense_fwd(int64_t m, int64_t n, const float4* __restrict__ X,
-            const float4* __restrict__ Y, int nrhs, const float* __restrict__ W,
-            float ns_log2e, float* __restrict__ out) {
-    __shared__ __align__(16) float Ks[kBN][kBM];
-    __shared__ __align__(16) float Ws[2][kBN][kRHS];
-    __shared__ float4 Ys[2][kBN];
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool live) {
+    const int sz = live ? 16 : 0;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(sz) : "memory");
+}
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src, bool live) {
+    const int sz = live ? 4 : 0;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(sz) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
+struct OwnArgs {
+    int64_t m, n;              // owned and other points
+    const float4* O;           // owned points
+    const float4* P;           // other points
+    int nrhs;                  // columns of A and B
+    const float* A;            // GRAD: weights of the owned points [m][nrhs]
+    const float* B;            // weights of the other points [n][nrhs]
+    float ns_log2e;            // -s log2(e)
+    float gscale;              // GRAD: factor of the written gradient (-2 s)
+    float* val;                // VAL: [m][nrhs], or the splits' partials [gridDim.y][m][nrhs]
+    float4* grad;              // GRAD: [m], or partials [gridDim.y][m] (may be NULL)
+    double* ds;                // GRAD: -sum e_o per block (may be NULL)
+};
+
+// R: columns a thread carries (a power of two); I: rows a thread owns (even).
+// gridDim = (row blocks, splits of the other points, column groups of R).
+template <int R, int I, bool VAL, bool GRAD, int OCC>
+__global__ void __launch_bounds__(kOwnThreads, OCC)
+k_dense_own(OwnArgs a) {
+    static_assert(I % 2 == 0 && (R & (R - 1)) == 0, "rows in pairs, columns a power of two");
+    constexpr int CH = R > 32 ? 64 : 128;     // points a stage
+    constexpr int NP = I / 2;                 // row pairs
+    constexpr int R2 = R > 1 ? R / 2 : 1;     // column pairs
+    __shared__ __align__(16) float4 Ys[2][CH];
+    __shared__ __align__(16) float Bs[2][CH * R];
+    // lets the combining kernel be scheduled early (it waits for this grid)
+    asm volatile("griddepcontrol.launch_dependents;");
+
     const int t = threadIdx.x;
-    const int tx = t & 15, ty = t >> 4;
-    const int64_t row0 = (int64_t)blockIdx.x * kBM;
-    // kernel-tile role: row r = t & 127 (its x in registers), 16 Y points
-    const int kr = t & (kBM - 1);
-    const int kh = t >> 7;  // 0 or 1: which 16 of the 32 Y points
-    float4 xi = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (row0 + kr < m) xi = __ldg(X + row0 + kr);
-    uint64_t acc2[4][4];   // acc2[p][c] = rows (ty*8 + 2p, ty*8 + 2p + 1), column tx*4 + c
+    const int64_t row0 = (int64_t)blockIdx.x * (kOwnThreads * I) + t;
+    const int c0 = blockIdx.z * R;
+    const int nc = a.nrhs - c0 < R ? a.nrhs - c0 : R;
+    const int64_t j_begin = a.n * blockIdx.y / gridDim.y;
+    const int64_t j_end = a.n * (blockIdx.y + 1) / gridDim.y;
+
+    uint64_t ox[NP], oy[NP], oz[NP];   // owned points, rows (2p, 2p + 1) packed
+    uint64_t av[GRAD ? I : 1][R2];     // GRAD: their weights (R = 1: in the low half)
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
+    for (int p = 0; p < NP; ++p) {
+        float4 o[2];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc2[p][c] = 0ull;
-    // W chunk: 32 x 64 floats, 8 per thread; Y chunk: 32 points
+        for (int u = 0; u < 2; ++u) {
+            const int64_t row = row0 + (2 * p + u) * kOwnThreads;
+            o[u] = row < a.m ? __ldg(a.O + row) : make_float4(0.f, 0.f, 0.f, 0.f);
+            if (GRAD) {
+#pragma unroll
+                for (int c = 0; c < R2; ++c) {
+                    const float* q = a.A + row * a.nrhs + 2 * c;
+                    const float lo = row < a.m && 2 * c < nc ? __ldg(q) : 0.f;
+                    const float hi = row < a.m && R > 1 && 2 * c + 1 < nc ? __ldg(q + 1) : 0.f;
+                    av[2 * p + u][c] = f2p(lo, hi);
+                }
+            }
+        }
+        ox[p] = f2p(o[0].x, o[1].x);
+        oy[p] = f2p(o[0].y, o[1].y);
+        oz[p] = f2p(o[0].z, o[1].z);
+    }
+    // sums: VAL per row and column pair (R = 1: per row pair); GRAD per row pair
+    uint64_t v[VAL ? (R > 1 ? I : NP) : 1][R2];
+    uint64_t gx[NP], gy[NP], gz[NP], ge[NP];
+#pragma unroll
+    for (int q = 0; q < (VAL ? (R > 1 ? I : NP) : 1); ++q)
+#pragma unroll
+        for (int c = 0; c < R2; ++c) v[q][c] = 0ull;
+#pragma unroll
+    for (int p = 0; p < NP; ++p) gx[p] = gy[p] = gz[p] = ge[p] = 0ull;
+
     auto stage = [&](int64_t j0, int b) {
-#pragma unroll
-        for (int e = 0; e < (kBN * kRHS) / kDThreads; ++e) {
-            const int idx = e * kDThreads + t;
-            const int jj = idx / kRHS, cc = idx % kRHS;
-            Ws[b][jj][cc] = (j0 + jj < n && cc < nrhs) ? __ldg(W + (j0 + jj) * nrhs + cc) : 0.f;
+        for (int q = t; q < CH; q += kOwnThreads) {
+            const bool live = j0 + q < j_end;
+            cp_async16((uint32_t)__cvta_generic_to_shared(&Ys[b][q]), a.P + (live ? j0 + q : 0), live);
         }
-        if (t < kBN) Ys[b][t] = (j0 + t < n) ? __ldg(Y + j0 + t) : make_float4(0.f, 0.f, 0.f, 0.f);
-    };
-    auto kernel_tile = [&](int64_t j0, int b) {
 #pragma unroll 4
-        for (int q = 0; q < 16; ++q) {
-            const int jj = kh * 16 + q;
-            const float4 y = Ys[b][jj];
-            const float dx = xi.x - y.x, dy = xi.y - y.y, dz = xi.z - y.z;
-            const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-            Ks[jj][kr] = (j0 + jj < n) ? ex2f(ns_log2e * d2) : 0.f;
+        for (int k = 0; k < CH * R / kOwnThreads; ++k) {
+            const int e = k * kOwnThreads + t;
+            const int jj = e / R, c = e % R;
+            const bool live = j0 + jj < j_end && c < nc;
+            cp_async4((uint32_t)__cvta_generic_to_shared(&Bs[b][e]),
+                      a.B + (live ? (j0 + jj) * a.nrhs + c0 + c : 0), live);
         }
+        cp_async_commit();
     };
-    const int64_t chunks = (n + kBN - 1) / kBN;
-    if (chunks > 0) {
-        stage(0, 0);
-        __syncthreads();
-        kernel_tile(0, 0);
-        __syncthreads();
+
+    const uint64_t ns2 = f2p(a.ns_log2e, a.ns_log2e);
+    int b = 0;
+    if (j_begin < j_end) stage(j_begin, 0);
+    for (int64_t j0 = j_begin; j0 < j_end; j0 += CH, b ^= 1) {
+        cp_async_wait_all();
+        __syncthreads();       // stage b is complete, and the other one fully read
+        if (j0 + CH < j_end) stage(j0 + CH, b ^ 1);
+        const int cnt = (int)(j_end - j0 < CH ? j_end - j0 : CH);
+        const float4* __restrict__ Yb = Ys[b];
+        const float* __restrict__ Bb = Bs[b];
+#pragma unroll (R >= 32 ? 1 : R >= 8 ? 2 : 4)
+        for (int j = 0; j < cnt; ++j) {
+            const float4 y = Yb[j];
+            const uint64_t yx = f2p(y.x, y.x), yy = f2p(y.y, y.y), yz = f2p(y.z, y.z);
+            uint64_t B2[R2];
+            if (R == 1) {
+                B2[0] = f2p(Bb[j], Bb[j]);
+            } else if (R == 2) {
+                B2[0] = *reinterpret_cast<const uint64_t*>(Bb + j * R);
+            } else {
+#pragma unroll
+                for (int c = 0; c < R2; c += 2) {
+                    const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(Bb + j * R + 2 * c);
+                    B2[c] = q.x;
+                    B2[c + 1 < R2 ? c + 1 : c] = q.y;
+                }
+            }
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                const uint64_t dx = fsub2(ox[p], yx), dy = fsub2(oy[p], yy), dz = fsub2(oz[p], yz);
+                const uint64_t d2 = ffma2(dz, dz, ffma2(dy, dy, fmul2(dx, dx)));
+                float e0, e1;
+                f2u(fmul2(d2, ns2), e0, e1);
+                const float k0 = ex2f(e0), k1 = ex2f(e1);
+                const uint64_t k2 = f2p(k0, k1);
+                if (VAL) {
+                    if (R == 1) {
+                        v[p][0] = ffma2(k2, B2[0], v[p][0]);
+                    } else {
+                        const uint64_t kk0 = f2p(k0, k0), kk1 = f2p(k1, k1);
+                        constexpr int q0 = 2;
+#pragma unroll
+                        for (int c = 0; c < R2; ++c) {
+                            v[R > 1 ? q0 * p : 0][c] = ffma2(kk0, B2[c], v[R > 1 ? q0 * p : 0][c]);
+                            v[R > 1 ? q0 * p + 1 : 0][c] = ffma2(kk1, B2[c], v[R > 1 ? q0 * p + 1 : 0][c]);
+                        }
+                    }
+                }
+                if (GRAD) {
+                    uint64_t S2;
+                    if (R == 1) {
+                        float w0, w1, a0, a1, z;
+                        f2u(B2[0], w0, w1);
+                        f2u(av[GRAD ? 2 * p : 0][0], a0, z);
+                        f2u(av[GRAD ? 2 * p + 1 : 0][0], a1, z);
+                        S2 = fmul2(f2p(a0, a1), f2p(w0, w1));
+                    } else {
+                        uint64_t s0 = 0ull, s1 = 0ull;
+#pragma unroll
+                        for (int c = 0; c < R2; ++c) {
+                            s0 = ffma2(av[GRAD ? 2 * p : 0][c], B2[c], s0);
+                            s1 = ffma2(av[GRAD ? 2 * p + 1 : 0][c], B2[c], s1);
+                        }
+                        float l0, h0, l1, h1;
+                        f2u(s0, l0, h0);
+                        f2u(s1, l1, h1);
+                        S2 = f2p(l0 + h0, l1 + h1);
+                    }
+                    const uint64_t A2 = fmul2(S2, k2);
+                    gx[p] = ffma2(A2, dx, gx[p]);
+                    gy[p] = ffma2(A2, dy, gy[p]);
+                    gz[p] = ffma2(A2, dz, gz[p]);
+                    ge[p] = ffma2(A2, d2, ge[p]);
+                }
+            }
+        }
     }
-    for (int64_t c = 0; c < chunks; ++c) {
-        const int b = (int)(c & 1);
+
+    double dsum = 0.0;
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        float x[2], y[2], z[2], e[2], w[2];
+        f2u(gx[p], x[0], x[1]);
+        f2u(gy[p], y[0], y[1]);
+        f2u(gz[p], z[0], z[1]);
+        f2u(ge[p], e[0], e[1]);
+        f2u(v[VAL && R == 1 ? p : 0][0], w[0], w[1]);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int64_t row = row0 + (2 * p + u) * kOwnThreads;
+            if (row >= a.m) continue;
+            if (VAL) {
+                float* q = a.val + ((int64_t)blockIdx.y * a.m + row) * a.nrhs + c0;
+                if (R == 1) {
+                    q[0] = w[u];
+                } else {
+#pragma unroll
+                    for (int c = 0; c < R2; ++c) {
+                        float lo, hi;
+                        f2u(v[R > 1 ? 2 * p + u : 0][c], lo, hi);
+                        if (2 * c < nc) q[2 * c] = lo;
+                        if (2 * c + 1 < nc) q[2 * c + 1] = hi;
+                    }
+                }
+            }
+            if (GRAD) {
+                if (a.grad)
+                    a.grad[(int64_t)blockIdx.y * a.m + row] =
+                        make_float4(a.gscale * x[u], a.gscale * y[u], a.gscale * z[u], 0.f);
+                dsum -= (double)e[u];
+            }
+        }
+    }
+    if (GRAD && a.ds) {   // FP64 block sum in a fixed order
+        __shared__ double s_red[kOwnThreads / 32];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) dsum += __shfl_down_sync(0xffffffffu, dsum, o);
+        if ((t & 31) == 0) s_red[t >> 5] = dsum;
+        __syncthreads();
+        if (t == 0) {
+            double tot = 0.0;
+#pragma unroll
+            for (int q = 0; q < kOwnThreads / 32; ++q) tot += s_red[q];
+            a.ds[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = tot;
+        }
+    }
+}
+
+// Sums of the splits' partials, in the order of the splits: `vals` floats and
+// `grads` float4 (either may be 0).
+__global__ void __launch_bounds__(256)
+k_dense_combine(int splits, int64_t vals, const float* __restrict__ pv, float* __restrict__ val,
+                int64_t grads, const float4* __restrict__ pg, float4* __restrict__ grad) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e < vals) {
+        float s = 0.f;
 #pragma unroll 8
-        for (int k = 0; k < kBN; ++k) {
-            const float4 a0 = *reinterpret_cast<const float4*>(&Ks[k][ty * 8]);
-            const float4 a1 = *reinterpret_cast<const float4*>(&Ks[k][ty * 8 + 4]);
-            const float4 w = *reinterpret_cast<const float4*>(&Ws[b][k][tx * 4]);
-            const uint64_t A[4] = {f2p(a0.x, a0.y), f2p(a0.z, a0.w), f2p(a1.x, a1.y), f2p(a1.z, a1.w)};
-            const uint64_t B[4] = {f2p(w.x, w.x), f2p(w.y, w.y), f2p(w.z, w.z), f2p(w.w, w.w)};
-#pragma unroll
-            for (int p = 0; p < 4; ++p)
-#pragma unroll
-                for (int cc = 0; cc < 4; ++cc) acc2[p][cc] = ffma2(A[p], B[cc], acc2[p][cc]);
+        for (int q = 0; q < splits; ++q) s += __ldcg(pv + q * vals + e);
+        val[e] = s;
+    } else if (e - vals < grads) {
+        const int64_t r = e - vals;
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+        for (int q = 0; q < splits; ++q) {
+            const float4 g = __ldcg(pg + q * grads + r);
+            s.x += g.x;
+            s.y += g.y;
+            s.z += g.z;
         }
-        __syncthreads();   // Ks and Ws[b] fully read
-        if (c + 1 < chunks) {
-            stage((c + 1) * kBN, b ^ 1);
-            __syncthreads();
-            kernel_tile((c + 1) * kBN, b ^ 1);
-            __syncthreads();
-        }
+        grad[r] = s;
     }
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-#pragma unroll
-        for (int cc = 0; cc < 4; ++cc) {
-            float v0, v1;
-            f2u(acc2[p][cc], v0, v1);
-            const int col = tx * 4 + cc;
-            const int64_t row = row0 + ty * 8 + 2 * p;
-            if (col < nrhs) {
-                if (row < m) out[row * nrhs + col] = v0;
-                if (row + 1 < m) out[(row + 1) * nrhs + col] = v1;
+}
+
+// Columns a thread carries, rows it owns and blocks per SM for a pass.
+struct OwnShape {
+    int R, I, occ;
+};
+
+// VAL alone: the cheapest power of two by its operations per pair (7 for the
+// distance and the exponent, one per column), counting the columns padded.
+// A gradient needs all columns in one thread: the next power of two.
+OwnShape own_shape(int nrhs, bool val, bool grad) {
+    if (!grad) {
+        int best = 32, cost = 1 << 30;
+        for (int R = 1; R <= 32; R *= 2) {
+            const int c = ((nrhs + R - 1) / R) * (7 + R);
+            if (c < cost) {
+                cost = c;
+                best = R;
             }
         }
+        return {best, 4, best >= 32 ? 2 : best >= 16 ? 3 : 4};
     }
+    int R = 1;
+    while (R < nrhs) R *= 2;
+    (void)val;
+    return {R, 2, R >= 32 ? 2 : R >= 16 ? 3 : 4};
 }
 
-// dX_i = -2 s (x_i sum_j A_ij - sum_j A_ij y_j), A_ij = (G_i . W_j) K_ij,
-// ds partial = -sum_ij A_ij d_ij^2 (one FP64 value per CTA).
-// Thread layout: row r = t & 127, j-half h = t >> 7 (16 Y points each).
-__global__ void __launch_bounds__(kDThreads)
-k_dense_gradx(int64_t m, int64_t n, const float4* __restrict__ X,
-              const float4* __restrict__ Y, int nrhs, const float* __restrict__ W,
-              const float* __restrict__ G, float s, float ns_log2e,
-              float4* __restrict__ dX, double* __restrict__ partial) {
-    __shared__ __align__(16) float Gs[kBM][kRHS + 4];   // padded rows
-    __shared__ __align__(16) float Ws[kBN][kRHS + 4];
-    __shared__ float4 Ys[kBN];
-
-    const int t = threadIdx.x;
-    const int r = t & (kBM - 1), h = t >> 7;
-    const int64_t row0 = (int64_t)blockIdx.x * kBM;
-    for (int e = t; e < kBM * kRHS; e += kDThreads) {
-        const int rr = e / kRHS, cc = e % kRHS;
-        Gs[rr][cc] = (row0 + rr < m && cc < nrhs) ? __ldg(G + (row0 + rr) * nrhs + cc) : 0.f;
-    }
-    float4 xi = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (row0 + r < m) xi = __ldg(X + row0 + r);
-    // accumulate A_ij (x_i - y_j) directly: no cancellation between
-    // x_i sum_j A_ij and sum_j A_ij y_j
-    float sX = 0.f, sY = 0.f, sZ = 0.f, sAd2 = 0.f;
-
-    for (int64_t j0 = 0; j0 < n; j0 += kBN) {
-        __syncthreads();
-        if (t < kBN) Ys[t] = (j0 + t < n) ? __ldg(Y + j0 + t) : make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int e = t; e < kBN * kRHS; e += kDThreads) {
-            const int jj = e / kRHS, cc = e % kRHS;
-            Ws[jj][cc] = (j0 + jj < n && cc < nrhs) ? __ldg(W + (j0 + jj) * nrhs + cc) : 0.f;
+// Splits of the n other points: the work of a block is its points plus about
+// 64 points' worth of start and write-out, and blocks run in waves of the
+// resident ones; the number of splits with the least time in that model.
+int plan_split(int64_t blocks, int64_t n, int occ) {
+    const int64_t resident = (int64_t)occ * num_sms();
+    int64_t most = (n + 63) / 64;
+    if (most > 256) most = 256;
+    int64_t best = 1, cost = INT64_MAX;
+    for (int64_t s = 1; s <= most; ++s) {
+        const int64_t waves = (blocks * s + resident - 1) / resident;
+        const int64_t c = waves * ((n + s - 1) / s + 64) + s / 4;
+        if (c < cost) {
+            cost = c;
+            best = s;
         }
-        __syncthreads();
-        // S_ij = G_i . W_j for this thread's row and 16 Y points
-        float S[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) S[q] = 0.f;
-#pragma unroll 4
-        for (int c = 0; c < kRHS; c += 4) {
-            const float4 gv = *reinterpret_cast<const float4*>(&Gs[r][c]);
-#pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const float4 wv = *reinterpret_cast<const float4*>(&Ws[h * 16 + q][c]);
-                S[q] = fmaf(gv.x, wv.x, fmaf(gv.y, wv.y, fmaf(gv.z, wv.z, fmaf(gv.w, wv.w, S[q]))));
+    }
+    return (int)best;
+}
+
+struct OwnPlan {
+    OwnShape sh;
+    int64_t blocks;   // row blocks
+    int groups;       // column groups
+    int splits;
+};
+
+OwnPlan own_plan(int64_t m, int64_t n, int nrhs, bool val, bool grad, bool may_split) {
+    OwnPlan p;
+    p.sh = own_shape(nrhs, val, grad);
+    const int64_t rows = (int64_t)kOwnThreads * p.sh.I;
+    p.blocks = (m + rows - 1) / rows;
+    p.groups = grad ? 1 : (nrhs + p.sh.R - 1) / p.sh.R;
+    p.splits = may_split ? plan_split(p.blocks * p.groups, n, p.sh.occ) : 1;
+    return p;
+}
+
+size_t own_bytes(const OwnPlan& p, int64_t m, int nrhs, bool val, bool grad) {
+    if (p.splits <= 1) return 0;
+    return (size_t)p.splits * m * ((val ? (size_t)nrhs * 4 : 0) + (grad ? 16 : 0)) + 32;
+}
+
+template <int R, bool VAL, bool GRAD>
+void own_launch(const OwnPlan& p, const OwnArgs& a, cudaStream_t st) {
+    constexpr int I = GRAD ? 2 : 4, OCC = R >= 32 ? 2 : R >= 16 ? 3 : 4;
+    const dim3 grid((unsigned)p.blocks, (unsigned)p.splits, (unsigned)p.groups);
+    k_dense_own<R, I, VAL, GRAD, OCC><<<grid, kOwnThreads, 0, st>>>(a);
+}
+
+template <bool VAL, bool GRAD>
+cudaError_t own_dispatch(const OwnPlan& p, const OwnArgs& a, cudaStream_t st) {
+    switch (p.sh.R) {
+        case 1: own_launch<1, VAL, GRAD>(p, a, st); break;
+        case 2: own_launch<2, VAL, GRAD>(p, a, st); break;
+        case 4: own_launch<4, VAL, GRAD>(p, a, st); break;
+        case 8: own_launch<8, VAL, GRAD>(p, a, st); break;
+        case 16: own_launch<16, VAL, GRAD>(p, a, st); break;
+        case 32: own_launch<32, VAL, GRAD>(p, a, st); break;
+        case 64:
+            if constexpr (GRAD && !VAL) {
+                own_launch<64, VAL, GRAD>(p, a, st);
+                break;
             }
-        }
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            const int jj = h * 16 + q;
-            if (j0 + jj >= n) continue;
-            const float4 y = Ys[jj];
-            const float dx = xi.x - y.x, dy = xi.y - y.y, dz = xi.z - y.z;
-            const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-            const float A = S[q] * ex2f(ns_log2e * d2);
-            sX = fmaf(A, dx, sX);
-            sY = fmaf(A, dy, sY);
-            sZ = fmaf(A, dz, sZ);
-            sAd2 = fmaf(A, d2, sAd2);
-        }
+            return cudaErrorInvalidValue;
+        default: return cudaErrorInvalidValue;
     }
-    __syncthreads();
-    // the W chunk buffer is free now: reuse it for the cross-half reduction
-    float (*red)[4] = reinterpret_cast<float (*)[4]>(&Ws[0][0]);
-    red[t][0] = sX; red[t][1] = sY; red[t][2] = sZ; red[t][3] = sAd2;
-    __syncthreads();
-    if (h == 0) {
-        const float ax = red[t][0] + red[t + kBM][0];
-        const float ay = red[t][1] + red[t + kBM][1];
-        const float az = red[t][2] + red[t + kBM][2];
-        const float ad = red[t][3] + red[t + kBM][3];
-        if (row0 + r < m && dX)
-            dX[row0 + r] = make_float4(-2.f * s * ax, -2.f * s * ay, -2.f * s * az, 0.f);
-        red[t][3] = ad;
-    }
-    __syncthreads();
-    if (t == 0 && partial) {
-        double tot = 0.0;
-        for (int q = 0; q < kBM; ++q) tot += (double)red[q][3];
-        partial[blockIdx.x] = -tot;
-    }
-}
-
-}  // namespace
-
-int dense_partial_capacity(int64_t m, int64_t n) {
-    (void)n;
-    return (int)((m + kBM - 1) / kBM);
-}
-
-cudaError_t launch_dense_fwd(int64_t m, int64_t n, const float4* X, const float4* Y,
-                             int nrhs, const float* W, float s, ab_prec prec,
-                             float* out, cudaStream_t st) {
-    if (m <= 0) return cudaSuccess;
-    if (prec != AB_PREC_FP32) return cudaErrorNotSupported;
-    const unsigned grid = (unsigned)((m + kBM - 1) / kBM);
-    k_dense_fwd<<<grid, kDThreads, 0, st>>>(m, n, X, Y, nrhs, W, -s * kLog2eD, out);
     return cudaGetLastError();
 }
 
+// One pass: values and / or gradients of the m owned points.  ws: the
+// splits' partials (own_bytes), or NULL to walk unsplit.  ds: per-block
+// partials, *ds_count of them.
+cudaError_t own_pass(int64_t m, int64_t n, const float4* O, const float4* P, int nrhs,
+                     const float* A, const float* B, float s, float* val, bool want_grad,
+                     float4* grad, double* ds, int* ds_count, void* ws, cudaStream_t st) {
+    const bool want_val = val != nullptr;
+    const OwnPlan p = own_plan(m, n, nrhs, want_val, want_grad, ws != nullptr);
+    OwnArgs a;
+    a.m = m;
+    a.n = n;
+    a.O = O;
+    a.P = P;
+    a.nrhs = nrhs;
+    a.A = A;
+    a.B = B;
+    a.ns_log2e = -s * kLog2eD;
+    a.gscale = -2.f * s;
+    a.val = val;
+    a.grad = grad;
+    a.ds = ds;
+    float4* pg = (float4*)ws;   // gradients first: 16-byte aligned
+    const int64_t ng = grad ? m : 0, nv = want_val ? m * nrhs : 0;
+    float* pv = (float*)(pg + (p.splits > 1 ? p.splits * ng : 0));
+    if (p.splits > 1) {
+        if (want_val) a.val = pv;
+        if (grad) a.grad = pg;
+    }
+    cudaError_t e = want_val ? (want_grad ? own_dispatch<true, true>(p, a, st)
+                                          : own_dispatch<true, false>(p, a, st))
+                             : own_dispatch<false, true>(p, a, st);
+    if (e != cudaSuccess) return e;
+    if (ds_count) *ds_count = (int)(p.blocks * p.splits);
+    if (p.splits > 1 && nv + ng > 0) {
+        // programmatic dependent launch: scheduled while the walk runs, waits
+        // in griddepcontrol.wait for its writes
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)((nv + ng + 255) / 256));
+        cfg.blockDim = dim3(256);
+        cfg.stream = st;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, k_dense_combine, p.splits, nv, (const float*)pv, val, ng,
+                               (const float4*)pg, grad);
+    }
+    return e;
+}
+
+// dW and dY share a walk while both fit a thread's registers.
+constexpr int kFusedRhs = 32;
+
+}  // namespace
+
+size_t dense_fwd_workspace_bytes(int64_t m, int64_t n, int nrhs) {
+    if (m <= 0 || n <= 0) return 0;
+    return own_bytes(own_plan(m, n, nrhs, true, false, true), m, nrhs, true, false);
+}
+
+size_t dense_bwd_workspace_bytes(int64_t m, int64_t n, int nrhs, bool dW, bool dX, bool dY, bool ds) {
+    size_t need = 0;
+    auto take = [&](int64_t rows, int64_t other, bool v, bool g) {
+        if (rows <= 0 || other <= 0) return;
+        const size_t b = own_bytes(own_plan(rows, other, nrhs, v, g, true), rows, nrhs, v, g);
+        if (b > need) need = b;
+    };
+    if (dX || ds) take(m, n, false, true);
+    if (dW && dY && nrhs <= kFusedRhs) {
+        take(n, m, true, true);
+    } else {
+        if (dW) take(n, m, true, false);
+        if (dY) take(n, m, false, true);
+    }
+    return need;
+}
+
+size_t dense_partial_capacity(int64_t m, int64_t n, int nrhs) {
+    if (m <= 0 || n <= 0) return 1;
+    const OwnPlan p = own_plan(m, n, nrhs, false, true, true);
+    return (size_t)(p.blocks * p.splits);
+}
+
+cudaError_t launch_dense_fwd(int64_t m, int64_t n, const float4* X, const float4* Y,
+                             int nrhs, const float* W, float s, float* out, void* ws,
+                             cudaStream_t st) {
+    if (m <= 0) return cudaSuccess;
+    if (n <= 0) return cudaMemsetAsync(out, 0, (size_t)m * nrhs * sizeof(float), st);
+    return own_pass(m, n, X, Y, nrhs, nullptr, W, s, out, false, nullptr, nullptr, nullptr, ws, st);
+}
+
 cudaError_t launch_dense_bwd(int64_t m, int64_t n, const float4* X, const float4* Y,
-                             int nrhs, const float* W, float s, ab_prec prec,
-                             const float* G, float* dW, float4* dX, float4* dY,
-                             double* partial, int* partial_count, cudaStream_t st) {
-    if (prec != AB_PREC_FP32) return cudaErrorNotSupported;
+                             int nrhs, const float* W, float s, const float* G, float* dW,
+                             float4* dX, float4* dY, double* partial, int* partial_count,
+                             void* ws, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
     *partial_count = 0;
-    if (dW && n > 0) {
-        const unsigned grid = (unsigned)((n + kBM - 1) / kBM);
-        k_dense_fwd<<<grid, kDThreads, 0, st>>>(n, m, Y, X, nrhs, G, -s * kLog2eD, dW);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (n > 0 && m <= 0) {
+        if (dW && (e = cudaMemsetAsync(dW, 0, (size_t)n * nrhs * sizeof(float), st)) != cudaSuccess) return e;
+        if (dY && (e = cudaMemsetAsync(dY, 0, (size_t)n * sizeof(float4), st)) != cudaSuccess) return e;
+        return e;
     }
-    if ((dX || partial) && m > 0) {
-        const unsigned grid = (unsigned)((m + kBM - 1) / kBM);
-        k_dense_gradx<<<grid, kDThreads, 0, st>>>(m, n, X, Y, nrhs, W, G, s, -s * kLog2eD,
-                                                  dX, partial);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if (partial) *partial_count = (int)grid;
+    if (m > 0 && n <= 0)
+        return dX ? cudaMemsetAsync(dX, 0, (size_t)m * sizeof(float4), st) : cudaSuccess;
+    if (m <= 0) return cudaSuccess;
+    if (dX || partial) {
+        e = own_pass(m, n, X, Y, nrhs, G, W, s, nullptr, true, dX, partial, partial_count, ws, st);
+        if (e != cudaSuccess) return e;
     }
-    if (dY && n > 0) {
-        const unsigned grid = (unsigned)((n + kBM - 1) / kBM);
-        k_dense_gradx<<<grid, kDThreads, 0, st>>>(n, m, Y, X, nrhs, G, W, s, -s * kLog2eD,
-                                                  dY, nullptr);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // K(X, Y)^T = K(Y, X): the columns own, the rows are walked
+    if (dW && dY && nrhs <= kFusedRhs)
+        return own_pass(n, m, Y, X, nrhs, W, G, s, dW, true, dY, nullptr, nullptr, ws, st);
+    if (dW) {
+        e = own_pass(n, m, Y, X, nrhs, nullptr, G, s, dW, false, nullptr, nullptr, nullptr, ws, st);
+        if (e != cudaSuccess) return e;
     }
-    return cudaSuccess;
+    if (dY) e = own_pass(n, m, Y, X, nrhs, W, G, s, nullptr, true, dY, nullptr, nullptr, ws, st);
+    return e;
 }
 
 }  // namespace ab

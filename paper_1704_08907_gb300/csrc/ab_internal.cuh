@@ -174,18 +174,22 @@ AB_HIDDEN cudaError_t launch_pair_count(const CellList& cl, uint32_t* counts,
 AB_HIDDEN cudaError_t launch_pair_emit(const CellList& cl, const int64_t* offsets,
                                        int32_t* idx, cudaStream_t st);
 
-// ab_dense.cu
+// ab_dense.cu (FP32 CUDA cores; ws: the bytes the *_workspace_bytes name, or
+// NULL: the walks are then not split over the other points)
+AB_HIDDEN size_t dense_fwd_workspace_bytes(int64_t m, int64_t n, int nrhs);
+AB_HIDDEN size_t dense_bwd_workspace_bytes(int64_t m, int64_t n, int nrhs, bool dW, bool dX,
+                                           bool dY, bool ds);
 AB_HIDDEN cudaError_t launch_dense_fwd(int64_t m, int64_t n, const float4* X,
                                        const float4* Y, int nrhs, const float* W,
-                                       float s, ab_prec prec, float* out,
-                                       cudaStream_t st);
+                                       float s, float* out, void* ws, cudaStream_t st);
 AB_HIDDEN cudaError_t launch_dense_bwd(int64_t m, int64_t n, const float4* X,
                                        const float4* Y, int nrhs, const float* W,
-                                       float s, ab_prec prec, const float* G,
+                                       float s, const float* G,
                                        float* dW, float4* dX, float4* dY,
-                                       double* partial, int* partial_count,
+                                       double* partial, int* partial_count, void* ws,
                                        cudaStream_t st);
-AB_HIDDEN int dense_partial_capacity(int64_t m, int64_t n);
+// ds partials of launch_dense_bwd
+AB_HIDDEN size_t dense_partial_capacity(int64_t m, int64_t n, int nrhs);
 
 // ab_dense_tc.cu (tcgen05 path; nrhs must be 64)
 AB_HIDDEN size_t dense_tc_workspace_bytes(int64_t n);
