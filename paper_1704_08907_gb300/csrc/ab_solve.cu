@@ -176,8 +176,14 @@ int solve_blocks(int64_t n) {
 
 }  // namespace
 
+// Floats a vector takes in the workspace: a multiple of 4, so that the FP64
+// partials that follow the vectors are aligned for every n and nrhs.
+static size_t solve_vector_floats(int64_t n, int nrhs) {
+    return ((size_t)n * nrhs + 3) & ~(size_t)3;
+}
+
 size_t solve_workspace_bytes(int64_t n, int nrhs) {
-    const size_t v = (size_t)n * nrhs * sizeof(float);
+    const size_t v = solve_vector_floats(n, nrhs) * sizeof(float);
     return 3 * v + (size_t)solve_blocks(n) * nrhs * sizeof(double) + (size_t)nrhs * sizeof(Col) +
            256 * 4;
 }
@@ -186,7 +192,7 @@ size_t solve_workspace_bytes(int64_t n, int nrhs) {
 cudaError_t run_solve(int64_t n, int nrhs, const float* B, float sigma2, float tol, int max_iter,
                       float* W, void* ws, const SolveMatvec& mv, int* iters, float* relres,
                       cudaStream_t st) {
-    const size_t v = (size_t)n * nrhs;
+    const size_t v = solve_vector_floats(n, nrhs);
     float* R = (float*)ws;
     float* P = R + v;
     float* Q = P + v;
