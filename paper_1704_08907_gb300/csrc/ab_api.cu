@@ -333,6 +333,8 @@ ab_status ab_sync(ab_ctx* c) {
             return fail(c, AB_ERR_TIMEOUT, "scan look-back wait exceeded its time limit");
         if (h & ab::DEVERR_TC_TIMEOUT)
             return fail(c, AB_ERR_TIMEOUT, "tensor-core pipeline wait exceeded its time limit");
+        if (h & ab::DEVERR_SOLVE_TIMEOUT)
+            return fail(c, AB_ERR_TIMEOUT, "solve grid barrier exceeded its time limit");
     }
     return AB_OK;
 }
@@ -736,24 +738,34 @@ ab_status ab_kernel_solve(ab_ctx* c, int64_t n, const float* X, int32_t nrhs, co
     if (n == 0) return AB_OK;
     ab::DeviceGuard dg(c->device);
     if (!dg.ok) return fail(c, AB_ERR_CUDA, "cannot make device %d current", c->device);
-    cudaError_t e = grow(&c->sc.solve_ws, &c->sc.cap_solve_ws, ab::solve_workspace_bytes(n, nrhs),
-                         c->stream);
-    void* ws = nullptr;
-    if (prec == AB_PREC_FP32) {
-        ws = dense_scratch(c, ab::dense_fwd_workspace_bytes(n, n, nrhs));
-    } else if (e == cudaSuccess) {
-        e = grow(&c->sc.dense_ws, &c->sc.cap_dense_ws, ab::dense_tc_workspace_bytes(n), c->stream);
-        ws = c->sc.dense_ws;
+    cudaError_t e;
+    int it = 0;
+    float rr = 0.0f;
+    if (prec == AB_PREC_FP32 && c->coop_launch && ab::solve_coop_supported(n, nrhs)) {
+        // without the memory for its slab, the stepwise form below
+        e = grow(&c->sc.solve_ws, &c->sc.cap_solve_ws, ab::solve_coop_workspace_bytes(n, nrhs), c->stream);
+        if (e == cudaSuccess) {
+            e = ab::run_solve_coop(n, nrhs, (const float4*)X, B, s, sigma2, tol, max_iter, W,
+                                   c->sc.solve_ws, &it, &rr, c->d_err, c->stream);
+            if (e == cudaSuccess) {
+                if (iters) *iters = it;
+                if (relres) *relres = rr;
+                return AB_OK;
+            }
+            if (e != cudaErrorNotSupported) return cuda_fail(c, e, "ab_kernel_solve");
+        }
     }
+    e = grow(&c->sc.solve_ws, &c->sc.cap_solve_ws, ab::solve_workspace_bytes(n, nrhs), c->stream);
+    if (e == cudaSuccess && prec != AB_PREC_FP32)
+        e = grow(&c->sc.dense_ws, &c->sc.cap_dense_ws, ab::dense_tc_workspace_bytes(n), c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "ab_kernel_solve workspace");
     const float4* X4 = (const float4*)X;
     const ab::SolveMatvec mv = [&](const float* P, float* Q) -> cudaError_t {
         if (prec == AB_PREC_FP32)
-            return ab::launch_dense_fwd(n, n, X4, X4, nrhs, P, s, Q, ws, c->stream);
-        return ab::launch_dense_tc_fwd(n, n, X4, X4, nrhs, P, s, prec, Q, ws, c->d_err, c->stream);
+            return ab::launch_dense_fwd_ordered(n, n, X4, X4, nrhs, P, s, Q, c->stream);
+        return ab::launch_dense_tc_fwd(n, n, X4, X4, nrhs, P, s, prec, Q, c->sc.dense_ws, c->d_err,
+                                       c->stream);
     };
-    int it = 0;
-    float rr = 0.0f;
     e = ab::run_solve(n, nrhs, B, sigma2, tol, max_iter, W, c->sc.solve_ws, mv, &it, &rr, c->stream);
     if (e == cudaErrorNotSupported)
         return fail(c, AB_ERR_UNSUPPORTED, "precision not available for this shape");

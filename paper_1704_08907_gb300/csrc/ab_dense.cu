@@ -327,6 +327,10 @@ k_dense_combine(int splits, int64_t vals, const float* __restrict__ pv, float* _
 }
 
 // Columns a thread carries, rows it owns and blocks per SM for a pass.
+// ORDERED values (the solve's product, whose iteration count follows the last
+// bits) keep one chain of FMAs per output over the points in increasing
+// index: no split, two rows a thread, and fewer columns a thread where that
+// brings more SMs to work (K is then evaluated once per column group).
 struct OwnShape {
     int R, I, occ;
 };
@@ -350,6 +354,26 @@ OwnShape own_shape(int nrhs, bool val, bool grad) {
     while (R < nrhs) R *= 2;
     (void)val;
     return {R, 2, R >= 32 ? 2 : R >= 16 ? 3 : 4};
+}
+
+OwnShape ordered_shape(int64_t m, int nrhs) {
+    OwnShape best = {1, 2, 4};
+    int64_t cost = INT64_MAX;
+    for (int R = 1; R <= 32; R *= 2) {
+        const int groups = (nrhs + R - 1) / R;
+        const int64_t blocks = (m + 2 * kOwnThreads - 1) / (2 * kOwnThreads) * groups;
+        // a block alone on its SM runs at the latency of its FMAs, about the
+        // time that two blocks take together
+        int64_t per_sm = (blocks + num_sms() - 1) / num_sms();
+        if (per_sm < 2) per_sm = 2;
+        const int64_t c = per_sm * (7 + R);
+        if (c < cost) {
+            cost = c;
+            best = {R, 2, R >= 32 ? 2 : R >= 16 ? 3 : 4};
+        }
+        if (R >= nrhs) break;
+    }
+    return best;
 }
 
 // Splits of the n other points: the work of a block is its points plus about
@@ -395,9 +419,15 @@ size_t own_bytes(const OwnPlan& p, int64_t m, int nrhs, bool val, bool grad) {
 
 template <int R, bool VAL, bool GRAD>
 void own_launch(const OwnPlan& p, const OwnArgs& a, cudaStream_t st) {
-    constexpr int I = GRAD ? 2 : 4, OCC = R >= 32 ? 2 : R >= 16 ? 3 : 4;
+    constexpr int OCC = R >= 32 ? 2 : R >= 16 ? 3 : 4;
     const dim3 grid((unsigned)p.blocks, (unsigned)p.splits, (unsigned)p.groups);
-    k_dense_own<R, I, VAL, GRAD, OCC><<<grid, kOwnThreads, 0, st>>>(a);
+    if constexpr (!GRAD) {
+        if (p.sh.I == 4) {
+            k_dense_own<R, 4, VAL, GRAD, OCC><<<grid, kOwnThreads, 0, st>>>(a);
+            return;
+        }
+    }
+    k_dense_own<R, 2, VAL, GRAD, OCC><<<grid, kOwnThreads, 0, st>>>(a);
 }
 
 template <bool VAL, bool GRAD>
@@ -510,6 +540,28 @@ cudaError_t launch_dense_fwd(int64_t m, int64_t n, const float4* X, const float4
     if (m <= 0) return cudaSuccess;
     if (n <= 0) return cudaMemsetAsync(out, 0, (size_t)m * nrhs * sizeof(float), st);
     return own_pass(m, n, X, Y, nrhs, nullptr, W, s, out, false, nullptr, nullptr, nullptr, ws, st);
+}
+
+cudaError_t launch_dense_fwd_ordered(int64_t m, int64_t n, const float4* X, const float4* Y,
+                                     int nrhs, const float* W, float s, float* out,
+                                     cudaStream_t st) {
+    if (m <= 0) return cudaSuccess;
+    if (n <= 0) return cudaMemsetAsync(out, 0, (size_t)m * nrhs * sizeof(float), st);
+    OwnPlan p;
+    p.sh = ordered_shape(m, nrhs);
+    p.blocks = (m + kOwnThreads * p.sh.I - 1) / (kOwnThreads * p.sh.I);
+    p.groups = (nrhs + p.sh.R - 1) / p.sh.R;
+    p.splits = 1;
+    OwnArgs a = {};
+    a.m = m;
+    a.n = n;
+    a.O = X;
+    a.P = Y;
+    a.nrhs = nrhs;
+    a.B = W;
+    a.ns_log2e = -s * kLog2eD;
+    a.val = out;
+    return own_dispatch<true, false>(p, a, st);
 }
 
 cudaError_t launch_dense_bwd(int64_t m, int64_t n, const float4* X, const float4* Y,

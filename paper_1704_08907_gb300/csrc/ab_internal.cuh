@@ -16,6 +16,7 @@ namespace ab {
 enum : uint32_t {
     DEVERR_SCAN_TIMEOUT = 1u,
     DEVERR_TC_TIMEOUT = 2u,   // a tensor-core kernel's pipeline wait gave up
+    DEVERR_SOLVE_TIMEOUT = 4u,   // a grid barrier of the one-launch solve gave up
 };
 
 // Cell-lattice geometry of one build, passed by value to kernels.
@@ -182,6 +183,10 @@ AB_HIDDEN size_t dense_bwd_workspace_bytes(int64_t m, int64_t n, int nrhs, bool 
 AB_HIDDEN cudaError_t launch_dense_fwd(int64_t m, int64_t n, const float4* X,
                                        const float4* Y, int nrhs, const float* W,
                                        float s, float* out, void* ws, cudaStream_t st);
+// each output one chain over the points in increasing index (the solve)
+AB_HIDDEN cudaError_t launch_dense_fwd_ordered(int64_t m, int64_t n, const float4* X,
+                                               const float4* Y, int nrhs, const float* W,
+                                               float s, float* out, cudaStream_t st);
 AB_HIDDEN cudaError_t launch_dense_bwd(int64_t m, int64_t n, const float4* X,
                                        const float4* Y, int nrhs, const float* W,
                                        float s, const float* G,
@@ -209,6 +214,13 @@ AB_HIDDEN size_t solve_workspace_bytes(int64_t n, int nrhs);
 AB_HIDDEN cudaError_t run_solve(int64_t n, int nrhs, const float* B, float sigma2, float tol,
                                 int max_iter, float* W, void* ws, const SolveMatvec& mv,
                                 int* iters, float* relres, cudaStream_t st);
+
+// The same in one cooperative launch (FP32, few columns)
+AB_HIDDEN bool solve_coop_supported(int64_t n, int nrhs);
+AB_HIDDEN size_t solve_coop_workspace_bytes(int64_t n, int nrhs);
+AB_HIDDEN cudaError_t run_solve_coop(int64_t n, int nrhs, const float4* X, const float* B, float s,
+                                     float sigma2, float tol, int max_iter, float* W, void* ws,
+                                     int* iters, float* relres, uint32_t* err, cudaStream_t st);
 
 // ab_bd.cu
 AB_HIDDEN cudaError_t launch_bd_step(const Geom& g, int64_t n, float4* pos,
