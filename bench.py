@@ -58,6 +58,16 @@ TRAFFIC_EG_BYTES = 35.54e6   # 29.28 MB read + 6.26 MB written
 TRAFFIC_SOURCE_SHA = "3b686070cc13ccc9"
 
 
+def pair_source_sha():
+    """Hash of the pair kernels' sources, which the traffic figures belong to."""
+    import hashlib
+    h = hashlib.sha256()
+    for name in ("ab_pairs.cuh", "ab_pairs.cu", "ab_pairs_grad.cu"):
+        with open(os.path.join(ROOT, "paper_1704_08907_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
+
+
 def alu_peak(pk):
     """FP32 lane-operations per second: SMs x 128 lanes x max SM clock, with
     the SM count read from the device."""
@@ -410,9 +420,7 @@ def run_ours(args, rank, world):
         e2e_value = pairs * args.steps / (e2e_ms * 1e-3)
         e2e_serial_value = pairs * args.steps / (e2e_serial_ms * 1e-3)
 
-    import hashlib
-    src = os.path.join(ROOT, "paper_1704_08907_gb300", "csrc", "ab_pairs.cu")
-    same_kernel = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16] == TRAFFIC_SOURCE_SHA
+    same_kernel = pair_source_sha() == TRAFFIC_SOURCE_SHA
     pk, pk_kind = peaks()
     alu, alu_src = alu_peak(pk)
     eg_ops = cands * OPS_PER_CANDIDATE + pairs * OPS_PER_PAIR_LJ_EG
@@ -684,9 +692,7 @@ def also_c3(reps=5, oracle_fraction=64):
     alu, alu_src = alu_peak(pk)
     fwd_ops = cands * OPS_PER_CANDIDATE + pairs * OPS_PER_PAIR_GAUSS_FWD
     bwd_ops = cands * OPS_PER_CANDIDATE + pairs * OPS_PER_PAIR_GAUSS_BWD
-    import hashlib
-    src = os.path.join(ROOT, "paper_1704_08907_gb300", "csrc", "ab_pairs.cu")
-    same = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16] == TRAFFIC_C3_SOURCE_SHA
+    same = pair_source_sha() == TRAFFIC_C3_SOURCE_SHA
     bbytes = build_bytes(w.n, ncells // int(np.prod(reach)))   # width-r cells
     out = {"workload": "16,777,216 points in 1024 Gaussian blobs, periodic cube, "
                        f"r={w.radius:.7f} (64 neighbours mean): rebuild + gauss fwd + adjoint",

@@ -20,9 +20,9 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libaboria_gpu.so")
-SOURCES = ["ab_api.cu", "ab_cells.cu", "ab_sort.cu", "ab_pairs.cu", "ab_dense.cu", "ab_dense_tc.cu", "ab_bd.cu",
+SOURCES = ["ab_api.cu", "ab_cells.cu", "ab_sort.cu", "ab_pairs.cu", "ab_pairs_grad.cu", "ab_dense.cu", "ab_dense_tc.cu", "ab_bd.cu",
            "ab_solve.cu"]
-HEADERS = [os.path.join(CSRC, "ab_internal.cuh"),
+HEADERS = [os.path.join(CSRC, "ab_internal.cuh"), os.path.join(CSRC, "ab_pairs.cuh"),
            os.path.join(ROOT, "include", "aboria_gpu.h"),
            os.path.join(ROOT, "include", "aboria_gpu_testing.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -512,7 +512,7 @@ ab_status ab_pair_sum(ab_ctx* c, ab_op op, const ab_op_params* prm, const float*
     ab::PairOut o;
     o.out = vec ? nullptr : out;
     o.out4 = vec ? (float4*)out : nullptr;
-    const int grid = ab::pair_grid(n);
+    const int grid = ab::pair_grid(c->cl);
     if (op == AB_OP_LJ && energy) {
         if ((s = ensure_partial(c, (size_t)grid)) != AB_OK) return s;
         o.partial = c->sc.partial;
@@ -550,7 +550,7 @@ static ab_status energy_grad_impl(ab_ctx* c, ab_op op, const ab_op_params* prm, 
     o.out = E;
     if (packed) o.grad_packed = grad;
     else o.grad_pos = (float4*)grad;
-    const int grid = ab::pair_grid(n);
+    const int grid = ab::pair_grid(c->cl);
     if (energy) {
         if ((s = ensure_partial(c, (size_t)grid)) != AB_OK) return s;
         o.partial = c->sc.partial;
@@ -616,7 +616,7 @@ static ab_status pair_bwd_impl(ab_ctx* c, ab_op op, const ab_op_params* prm, con
     o.grad_pos = (float4*)grad_pos4;
     o.grad_w = op == AB_OP_GAUSS ? grad_w : nullptr;
     o.out = value ? out : nullptr;
-    const int grid = ab::pair_grid(n);
+    const int grid = ab::pair_grid(c->cl);
     double* red = op == AB_OP_GAUSS ? grad_s : (value ? energy : nullptr);
     if (red) {
         if ((s = ensure_partial(c, (size_t)grid)) != AB_OK) return s;
