@@ -417,8 +417,11 @@ static ab_status build_impl(ab_ctx* c, const ab_domain* dom, int64_t n, const fl
     if (s != AB_OK) return s;
     if (!c->sc.coop) {
         e = cudaMallocAsync((void**)&c->sc.coop, ab::coop_scratch_words() * sizeof(uint32_t), c->stream);
+        if (e == cudaSuccess)
+            e = cudaMemsetAsync(c->sc.coop, 0, ab::coop_scratch_words() * sizeof(uint32_t), c->stream);
         if (e != cudaSuccess) {
             cudaGetLastError();
+            if (c->sc.coop) cudaFreeAsync(c->sc.coop, c->stream);
             c->sc.coop = nullptr;
             return cuda_fail(c, e, "ab_build (build scratch)");
         }

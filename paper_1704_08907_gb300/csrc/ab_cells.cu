@@ -307,6 +307,7 @@ k_reduce_partials(const double* __restrict__ partial, int count, double* __restr
 // sorted order is the dense table's bit for bit.
 // ---------------------------------------------------------------------------
 constexpr int kCoopThreads = 1024;
+constexpr int kCoopBarWords = 4;        // barrier words at the start of the scratch (zeroed once)
 constexpr int kCoopIlp = 4;             // particles per thread per loop trip
 constexpr int kCoopScanItems = 16;      // cells per thread per scan tile (4 x 16-byte loads)
 
@@ -323,7 +324,7 @@ struct CoopArgs {
     uint32_t* perm;
     float4* spos;
     uint32_t* block_sum;       // [gridDim.x]
-    uint32_t* bar;             // [2]: arrivals, generation (zero at launch)
+    uint32_t* bar;             // [3]: arrivals, generation, blocks done (see coop_exit)
     uint32_t* err;
     long long limit_ns;
     int skip_block;            // testing: this block never arrives at the first barrier (-1: none)
@@ -355,6 +356,20 @@ __device__ __forceinline__ void coop_barrier(uint32_t* bar, uint32_t* err, long 
         __threadfence();
     }
     __syncthreads();
+}
+
+// At the end of a cooperative launch: the last block to get here resets the
+// arrivals, so that a launch whose waits ran out leaves the barrier clean for
+// the next one (a launch used to clear it with a memset of its own before
+// it).  Every block gets here: all waits are bounded.
+__device__ __forceinline__ void coop_exit(uint32_t* bar) {
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(bar + 2, 1u) == gridDim.x - 1) {
+            bar[0] = 0u;
+            bar[2] = 0u;
+        }
+    }
 }
 
 __device__ __forceinline__ uint32_t ldcg_u32(const uint32_t* p) { return __ldcg(p); }
@@ -658,6 +673,7 @@ k_build_coop(CoopArgs a) {
     coop_scatter(a, tid, nthreads);
     coop_barrier(a.bar, a.err, a.limit_ns);
     coop_finalize<DIM, PACKED>(a, tid, nthreads);
+    coop_exit(a.bar);
 }
 
 template <int DIM, bool PACKED>
@@ -759,6 +775,78 @@ k_build_coop_compact(CoopArgs a) {
     coop_scatter_idx(a, idx32, tid, nthreads);
     coop_barrier(a.bar, a.err, a.limit_ns);
     coop_finalize_idx<DIM, PACKED>(a, idx32, tid, nthreads);
+    coop_exit(a.bar);
+}
+
+// The whole build in one block, for few particles and cells: counts, offsets
+// and unordered slots live in shared memory and each thread keeps its
+// particles' positions in registers, so the caller's array is read once,
+// nothing is gathered and the phases are separated by block barriers.  The
+// same cell list as the other forms, bit for bit.  Bound: launch and the
+// latency of one round trip to memory; the cooperative form pays five grid
+// barriers and as many trips to L2 (1,000 points 20.6 -> 3.8 us, 4,096 27 -> 9,
+// 8,192 29 -> 16).
+template <int DIM, bool PACKED, int PER>
+__global__ void __launch_bounds__(kCoopThreads, 1)
+k_build_small(CoopArgs a) {
+    asm volatile("griddepcontrol.launch_dependents;");
+    extern __shared__ __align__(16) uint32_t s_dyn[];
+    __shared__ uint32_t s_warp[32];
+    const int n = (int)a.n, nc1 = (int)a.nc1, t = threadIdx.x;
+    uint32_t* s_start = s_dyn;                                  // [nc1]: counts, then offsets
+    uint32_t* s_slot = s_dyn + ((nc1 + 3) & ~3);                // [n]: original index per slot
+    for (int c = t; c < nc1; c += kCoopThreads) s_start[c] = 0u;
+    float4 q[PER];
+    uint32_t cell[PER], rank[PER];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const int i = u * kCoopThreads + t;
+        q[u] = i < n ? load_pos<DIM, PACKED>(a.pos, i) : make_float4(0.f, 0.f, 0.f, 0.f);
+        cell[u] = particle_cell<DIM, PACKED>(a, q[u]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < PER; ++u)
+        if (u * kCoopThreads + t < n) rank[u] = atomicAdd(s_start + cell[u], 1u);
+    __syncthreads();
+    {   // counts -> offsets: a run of entries per thread
+        const int per = (nc1 + kCoopThreads - 1) / kCoopThreads;
+        const int c0 = t * per, c1 = c0 + per < nc1 ? c0 + per : nc1;
+        uint32_t sum = 0, total;
+        for (int c = c0; c < c1; ++c) sum += s_start[c];
+        uint32_t ex = block_excl_scan(sum, s_warp, &total);
+        for (int c = c0; c < c1; ++c) {
+            const uint32_t v = s_start[c];
+            s_start[c] = ex;
+            ex += v;
+        }
+    }
+    __syncthreads();
+    for (int c = t; c < nc1; c += kCoopThreads) a.cell_start[c] = s_start[c];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const int i = u * kCoopThreads + t;
+        if (i < n) s_slot[s_start[cell[u]] + rank[u]] = (uint32_t)i;
+    }
+    __syncthreads();
+    // stable rank: the members of the cell with a smaller original index
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const int i = u * kCoopThreads + t;
+        if (i >= n) continue;
+        const uint32_t lo = s_start[cell[u]], hi = s_start[cell[u] + 1];
+        uint32_t r = 0, s = lo;
+        if (hi - lo >= 16) {            // crowded cells: four members a load
+            for (; s & 3u; ++s) r += s_slot[s] < (uint32_t)i ? 1u : 0u;
+            for (; s + 4 <= hi; s += 4) {
+                const uint4 m = *reinterpret_cast<const uint4*>(s_slot + s);
+                r += (m.x < (uint32_t)i) + (m.y < (uint32_t)i) + (m.z < (uint32_t)i) + (m.w < (uint32_t)i);
+            }
+        }
+        for (; s < hi; ++s) r += s_slot[s] < (uint32_t)i ? 1u : 0u;
+        a.perm[lo + r] = (uint32_t)i;
+        a.spos[lo + r] = make_float4(q[u].x, q[u].y, DIM == 3 ? q[u].z : 0.0f, 0.0f);
+    }
 }
 
 // Dense offsets of a compact cell list (inspection and export).
@@ -837,12 +925,15 @@ static int coop_grid(const void* fn, int64_t n, int64_t nc1) {
     }
     const int64_t resident = (int64_t)per_sm * num_sms();
     const int64_t work = n > nc1 ? n : nc1;
-    int64_t want = (work + (int64_t)kCoopThreads * kCoopIlp - 1) / ((int64_t)kCoopThreads * kCoopIlp);
+    // a block for every 1024 particles or cells: on a part of the chip each
+    // phase is a chain of L2 round trips (a quarter of the blocks measured
+    // 32 / 63 us at 262,144 points / 65,536 in 576 cells, against 27 / 37)
+    int64_t want = (work + kCoopThreads - 1) / kCoopThreads;
     if (want < 1) want = 1;
     return (int)(want < resident ? want : resident);
 }
 
-size_t coop_scratch_words() { return 2 + 4096; }   // barrier words + block sums
+size_t coop_scratch_words() { return kCoopBarWords + 4096; }   // barrier words + block sums
 
 // The counting sort in one launch where the device allows it (the kernel
 // sequence above 2^21 particles with a dense table).  The radix sort of
@@ -853,6 +944,32 @@ int auto_build_path(int64_t n, const Geom& g) {
     (void)n;
     (void)g;
     return kPathCoop;
+}
+
+// Particles and shared memory (offsets and slots) up to which the one-block
+// build is taken (8,192 points: 16 us against the cooperative form's 21).
+constexpr int64_t kSmallMaxN = 8192;
+constexpr size_t kSmallMaxSmem = 128 * 1024;
+
+static size_t small_smem(int64_t n, int64_t nc1) {
+    return (size_t)(((nc1 + 3) & ~(int64_t)3) + n) * sizeof(uint32_t);
+}
+
+template <int DIM, bool PACKED>
+static cudaError_t launch_small(const CoopArgs& a, cudaStream_t st) {
+    const size_t smem = small_smem(a.n, a.nc1);
+    auto go = [&](void (*kern)(CoopArgs)) -> cudaError_t {
+        if (smem > 48 * 1024) {   // per device: set on every such launch
+            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)kSmallMaxSmem);
+            if (e != cudaSuccess) return e;
+        }
+        kern<<<1, kCoopThreads, smem, st>>>(a);
+        return cudaGetLastError();
+    };
+    return a.n <= kCoopThreads       ? go(k_build_small<DIM, PACKED, 1>)
+           : a.n <= 4 * kCoopThreads ? go(k_build_small<DIM, PACKED, 4>)
+                                     : go(k_build_small<DIM, PACKED, 8>);
 }
 
 cudaError_t launch_build(CellList& cl, const float* pos, bool packed, Scratch& sc,
@@ -871,6 +988,19 @@ cudaError_t launch_build(CellList& cl, const float* pos, bool packed, Scratch& s
     const int path = opt.path == kPathAuto ? auto_build_path(n, cl.g) : opt.path;
     if (path == kPathRadix && radix_supported(n, nc))
         return launch_build_radix(cl, pos, packed, sc, err, st, opt);
+    if (!compact && opt.path == kPathAuto && opt.skip_block < 0 && n <= kSmallMaxN &&
+        small_smem(n, nc + 1) <= kSmallMaxSmem) {
+        CoopArgs a = {};
+        a.pos = pos;
+        a.n = n;
+        a.g = cl.g;
+        a.nc1 = nc + 1;
+        a.cell_start = cl.cell_start;
+        a.perm = cl.perm;
+        a.spos = cl.spos;
+        if (cl.g.dim == 3) return packed ? launch_small<3, true>(a, st) : launch_small<3, false>(a, st);
+        return packed ? launch_small<2, true>(a, st) : launch_small<2, false>(a, st);
+    }
     if (sc.coop && (compact || (path != kPathSequence && n <= kSingleLaunchMaxN))) {
         const void* fn;
         if (compact) {
@@ -896,14 +1026,12 @@ cudaError_t launch_build(CellList& cl, const float* pos, bool packed, Scratch& s
             a.perm = cl.perm;
             a.spos = cl.spos;
             a.bar = sc.coop;
-            a.block_sum = sc.coop + 2;
+            a.block_sum = sc.coop + kCoopBarWords;
             a.err = err;
             a.limit_ns = opt.limit_ns > 0 ? opt.limit_ns : kScanLimitNs;
             a.skip_block = opt.skip_block < grid ? opt.skip_block : -1;
-            cudaError_t e = cudaMemsetAsync(sc.coop, 0, 2 * sizeof(uint32_t), st);
-            if (e != cudaSuccess) return e;
             void* args[] = {&a};
-            e = cudaLaunchCooperativeKernel(fn, dim3((unsigned)grid), dim3(kCoopThreads), args, 0, st);
+            cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3((unsigned)grid), dim3(kCoopThreads), args, 0, st);
             if (e == cudaSuccess || compact) return e;
             cudaGetLastError();   // not launchable here: fall back to the kernel sequence
         }
