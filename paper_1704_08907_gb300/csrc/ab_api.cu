@@ -611,9 +611,9 @@ static ab_status pair_bwd_impl(ab_ctx* c, ab_op op, const ab_op_params* prm, con
     cudaError_t e;
     if ((s = ensure_sv(c, n)) != AB_OK) return s;
     // g into the pad of the sorted positions; GAUSS also needs w, as float[n]
-    e = ab::launch_gather_w_pos(c->cl, grad_out, c->stream);
-    if (e == cudaSuccess && op == AB_OP_GAUSS)
-        e = ab::launch_gather_scalar(c->cl, w, reinterpret_cast<float*>(c->sc.sv), c->stream);
+    e = op == AB_OP_GAUSS ? ab::launch_gather_pad_scalar(c->cl, grad_out, w,
+                                                         reinterpret_cast<float*>(c->sc.sv), c->stream)
+                          : ab::launch_gather_w_pos(c->cl, grad_out, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "adjoint gather");
     ab::PairOut o;
     o.grad_pos = (float4*)grad_pos4;

@@ -4,6 +4,7 @@
 // r_cut).  Everything is HBM-bound element-wise work: float4 coalesced loads,
 // grid-stride loops sized to the SM count, a single-pass decoupled look-back
 // scan with bounded waits.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -262,31 +263,53 @@ k_scan(const uint32_t* in, TOut* out, int64_t n, uint64_t* status,
     }
 }
 
-constexpr int kRedThreads = 1024;
+// Sum of FP64 partials in a fixed order, by one cluster: each block a
+// contiguous share (four chains a thread, shuffles, warps in order), the
+// blocks' sums meeting in the first one's shared memory.  Bound: the FP64
+// pipe, 16 clocks and more a warp addition and SM (one block of 1024 threads
+// with a shared-memory tree: the 1M-point LJ call with its 8,192 partials 270
+// us, so 266; 131,072 partials alone 44 us).
+constexpr int kRedThreads = 256;
+constexpr int kRedBlocks = 8;
 __global__ void __launch_bounds__(kRedThreads)
 k_reduce_partials(const double* __restrict__ partial, int count, double* __restrict__ out) {
     // launched as a programmatic dependent of the kernel that writes the
     // partials: wait until that grid has finished and its writes are visible
     // (returns at once without a prerequisite grid)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    // fixed assignment and tree order: deterministic for a given count
-    __shared__ double s[kRedThreads];
+    __shared__ double s_warp[kRedThreads / 32];
+    __shared__ double s_block[kRedBlocks];
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int blocks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int share = (count + blocks - 1) / blocks;
+    const int end = min(count, (rank + 1) * share);
     double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-    int t = threadIdx.x;
-    for (; t + 3 * kRedThreads < count; t += 4 * kRedThreads) {
+    int t = rank * share + (int)threadIdx.x;
+    for (; t + 3 * kRedThreads < end; t += 4 * kRedThreads) {
         a0 += partial[t];
         a1 += partial[t + kRedThreads];
         a2 += partial[t + 2 * kRedThreads];
         a3 += partial[t + 3 * kRedThreads];
     }
-    for (; t < count; t += kRedThreads) a0 += partial[t];
-    s[threadIdx.x] = (a0 + a1) + (a2 + a3);
+    for (; t < end; t += kRedThreads) a0 += partial[t];
+    double v = (a0 + a1) + (a2 + a3);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = v;
     __syncthreads();
-    for (int w = kRedThreads / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) s[threadIdx.x] += s[threadIdx.x + w];
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        double b = 0.0;
+#pragma unroll
+        for (int w = 0; w < kRedThreads / 32; ++w) b += s_warp[w];
+        *cluster.map_shared_rank(&s_block[rank], 0) = b;
     }
-    if (threadIdx.x == 0) *out = s[0];
+    cluster.sync();
+    if (rank == 0 && threadIdx.x == 0) {
+        double sum = 0.0;
+        for (int b = 0; b < blocks; ++b) sum += s_block[b];
+        *out = sum;
+    }
 }
 
 
@@ -903,14 +926,19 @@ cudaError_t launch_reduce_partials(const double* partial, int count, double* out
     // launch_dependents at their start) and waits in griddepcontrol.wait, so
     // its launch latency is hidden
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(1);
+    const unsigned blocks = count > 4 * kRedThreads ? kRedBlocks : 1;
+    cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(kRedThreads);
     cfg.stream = st;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = blocks;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, k_reduce_partials, partial, count, out);
 }
 
@@ -1087,9 +1115,33 @@ k_gather_scalar(int64_t n, const uint32_t* __restrict__ perm, const float* __res
         out[s] = __ldg(v + perm[s]);
 }
 
-cudaError_t launch_gather_scalar(const CellList& cl, const float* v, float* out, cudaStream_t st) {
+// Two per-particle scalars in one pass over the permutation: g into the pad of
+// the sorted positions, w as out[s] = w[perm[s]].
+__global__ void __launch_bounds__(kThreads)
+k_gather_pad_scalar(int64_t n, const uint32_t* __restrict__ perm, const float* __restrict__ g,
+                    const float* __restrict__ w, float4* __restrict__ spos, float* __restrict__ out) {
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n;
+         s += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t p = perm[s];
+        const float gs = __ldg(g + p), ws = __ldg(w + p);
+        spos[s].w = gs;
+        out[s] = ws;
+    }
+}
+
+cudaError_t launch_gather_pad_scalar(const CellList& cl, const float* g, const float* w, float* out,
+                                     cudaStream_t st) {
     if (cl.n <= 0) return cudaSuccess;
-    k_gather_scalar<<<ew_grid(cl.n), kThreads, 0, st>>>(cl.n, cl.perm, v, out);
+    // one pass saves a launch, but its random reads need both arrays in L2:
+    // at 16.7M points (2 x 67 MB) it took 400 us against 142 + 81 apart
+    constexpr int64_t kOnePassMaxN = int64_t(1) << 22;
+    const int grid = ew_grid(cl.n);
+    if (cl.n <= kOnePassMaxN) {
+        k_gather_pad_scalar<<<grid, kThreads, 0, st>>>(cl.n, cl.perm, g, w, cl.spos, out);
+    } else {
+        k_gather_w_pos<<<grid, kThreads, 0, st>>>(cl.n, cl.perm, g, cl.spos);
+        k_gather_scalar<<<grid, kThreads, 0, st>>>(cl.n, cl.perm, w, out);
+    }
     return cudaGetLastError();
 }
 

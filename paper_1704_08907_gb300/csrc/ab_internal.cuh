@@ -125,8 +125,9 @@ AB_HIDDEN cudaError_t launch_build_radix(CellList& cl, const float* pos, bool pa
 // c = 0 .. n_cells (device uint32[n_cells + 1]).
 AB_HIDDEN cudaError_t launch_expand_cells(const CellList& cl, uint32_t* out, cudaStream_t st);
 AB_HIDDEN cudaError_t launch_gather_w_pos(CellList& cl, const float* w, cudaStream_t st);
-AB_HIDDEN cudaError_t launch_gather_scalar(const CellList& cl, const float* v, float* out,
-                                           cudaStream_t st);
+// g into the pad of the sorted positions and out[s] = w[perm[s]]
+AB_HIDDEN cudaError_t launch_gather_pad_scalar(const CellList& cl, const float* g, const float* w,
+                                               float* out, cudaStream_t st);
 // sv[s] = wv[perm[s]]: a per-particle pair of values into sorted order
 AB_HIDDEN cudaError_t launch_gather_pairs(const CellList& cl, const float2* wv, float2* sv,
                                           cudaStream_t st);
