@@ -68,7 +68,7 @@ def OpParams(s=0.0, eps=1.0, sigma=1.0, c=1.0, k=1.0) -> _abi.ab_op_params:
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _dev(t, dtype, shape_tail=None, name="tensor"):
@@ -80,9 +80,16 @@ def _dev(t, dtype, shape_tail=None, name="tensor"):
         raise TypeError(f"{name} must be {dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if shape_tail is not None and tuple(t.shape[1:]) != tuple(shape_tail):
+    if shape_tail is not None and t.shape[1:] != shape_tail:
         raise ValueError(f"{name} must have shape [n, {shape_tail}]")
     return t
+
+
+def _stream_of(device_index):
+    return torch.cuda.current_stream(device_index).cuda_stream
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", _stream_of)
 
 
 class Context:
@@ -99,7 +106,8 @@ class Context:
         self.build_seq = 0
 
     def _stream(self):
-        _lib.ab_set_stream(self.handle, ctypes.c_void_p(torch.cuda.current_stream(self.device).cuda_stream))
+        # the raw handle: a torch.cuda.Stream object for each call costs 2 us
+        _lib.ab_set_stream(self.handle, _raw_stream(self.device.index))
 
     def close(self):
         if getattr(self, "handle", None):

@@ -2,6 +2,8 @@
 
 The backward passes call the library's hand-written adjoint kernels, which
 recompute the pairs from the cell list instead of storing a neighbour list.
+Only data pointers leave these functions, so inputs are passed on as they are
+(a detached copy of each would cost the host a few microseconds a call).
 """
 from __future__ import annotations
 
@@ -27,7 +29,7 @@ class LJEnergy(torch.autograd.Function):
 
     @staticmethod
     def forward(fctx, pos4, abctx, dom, eps, sigma, energy=None):
-        seq = ab_build(abctx, dom, pos4.detach())
+        seq = ab_build(abctx, dom, pos4)
         prm = OpParams(eps=eps, sigma=sigma)
         E = ab_pair_sum(abctx, AB_OP_LJ, prm, energy=energy)
         fctx.save_for_backward(pos4)
@@ -37,7 +39,7 @@ class LJEnergy(torch.autograd.Function):
     @staticmethod
     def backward(fctx, gE):
         (pos4,) = fctx.saved_tensors
-        _ensure_built(fctx.abctx, fctx.dom, pos4.detach(), fctx.seq)
+        _ensure_built(fctx.abctx, fctx.dom, pos4, fctx.seq)
         g = torch.empty_like(pos4)
         ab_pair_sum_bwd(fctx.abctx, AB_OP_LJ, fctx.prm, None, gE.contiguous(), grad_pos4=g)
         return g, None, None, None, None, None
@@ -50,9 +52,9 @@ class GaussPairSum(torch.autograd.Function):
     @staticmethod
     def forward(fctx, pos4, w, s, abctx, dom):
         sval = float(s)
-        seq = ab_build(abctx, dom, pos4.detach())
+        seq = ab_build(abctx, dom, pos4)
         prm = OpParams(s=sval)
-        y = ab_pair_sum(abctx, AB_OP_GAUSS, prm, w=w.detach().contiguous())
+        y = ab_pair_sum(abctx, AB_OP_GAUSS, prm, w=w.contiguous())
         fctx.save_for_backward(pos4, w)
         fctx.abctx, fctx.dom, fctx.prm, fctx.seq = abctx, dom, prm, seq
         fctx.s_is_tensor = isinstance(s, torch.Tensor)
@@ -61,13 +63,15 @@ class GaussPairSum(torch.autograd.Function):
     @staticmethod
     def backward(fctx, gy):
         pos4, w = fctx.saved_tensors
-        _ensure_built(fctx.abctx, fctx.dom, pos4.detach(), fctx.seq)
+        _ensure_built(fctx.abctx, fctx.dom, pos4, fctx.seq)
         gpos = torch.empty_like(pos4)
         gw = torch.empty_like(w)
-        gs = torch.empty((), dtype=torch.float64, device=pos4.device)
-        ab_pair_sum_bwd(fctx.abctx, AB_OP_GAUSS, fctx.prm, w.detach().contiguous(),
+        # ds costs a reduction of its own: only when s is differentiated
+        gs = (torch.empty((), dtype=torch.float64, device=pos4.device) if fctx.s_is_tensor
+              else None)
+        ab_pair_sum_bwd(fctx.abctx, AB_OP_GAUSS, fctx.prm, w.contiguous(),
                         gy.contiguous(), grad_pos4=gpos, grad_w=gw, grad_s=gs)
-        return gpos, gw, (gs if fctx.s_is_tensor else None), None, None
+        return gpos, gw, gs, None, None
 
 
 class KernelMatvec(torch.autograd.Function):
@@ -76,7 +80,7 @@ class KernelMatvec(torch.autograd.Function):
     @staticmethod
     def forward(fctx, X, Y, W, s, abctx, prec="fp32"):
         sval = float(s)
-        out = ab_kernel_matvec(abctx, X.detach(), Y.detach(), W.detach().contiguous(), sval, prec)
+        out = ab_kernel_matvec(abctx, X, Y, W.contiguous(), sval, prec)
         fctx.save_for_backward(X, Y, W)
         fctx.abctx, fctx.sval, fctx.prec = abctx, sval, prec
         fctx.s_is_tensor = isinstance(s, torch.Tensor)
@@ -89,7 +93,7 @@ class KernelMatvec(torch.autograd.Function):
         dX = torch.empty_like(X) if fctx.needs_input_grad[0] else None
         dY = torch.empty_like(Y) if fctx.needs_input_grad[1] else None
         ds = torch.empty((), dtype=torch.float64, device=X.device) if fctx.s_is_tensor else None
-        ab_kernel_matvec_bwd(fctx.abctx, X.detach(), Y.detach(), W.detach().contiguous(),
+        ab_kernel_matvec_bwd(fctx.abctx, X, Y, W.contiguous(),
                              fctx.sval, fctx.prec, G.contiguous(), dW=dW, dX=dX, dY=dY, ds=ds)
         return dX, dY, dW, ds, None, None
 
