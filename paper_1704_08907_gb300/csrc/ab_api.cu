@@ -711,9 +711,10 @@ ab_status ab_kernel_matvec(ab_ctx* c, int64_t m, int64_t n, const float* X, cons
     } else {
         if (nrhs != 64)
             return fail(c, AB_ERR_UNSUPPORTED, "tensor-core paths need nrhs == 64");
-        e = grow(&c->sc.dense_ws, &c->sc.cap_dense_ws, ab::dense_tc_workspace_bytes(n), c->stream);
+        e = grow(&c->sc.dense_ws, &c->sc.cap_dense_ws, ab::dense_tc_workspace_bytes(m, n, prec, false),
+                 c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "ab_kernel_matvec workspace");
-        e = ab::launch_dense_tc_fwd(m, n, (const float4*)X, (const float4*)Y, nrhs, W, s, prec, out,
+        e = ab::launch_dense_tc_fwd(m, n, (const float4*)X, (const float4*)Y, nrhs, W, s, prec, out, false,
                                     c->sc.dense_ws, c->d_err, c->stream);
     }
     if (e == cudaErrorNotSupported)
@@ -760,13 +761,14 @@ ab_status ab_kernel_solve(ab_ctx* c, int64_t n, const float* X, int32_t nrhs, co
     }
     e = grow(&c->sc.solve_ws, &c->sc.cap_solve_ws, ab::solve_workspace_bytes(n, nrhs), c->stream);
     if (e == cudaSuccess && prec != AB_PREC_FP32)
-        e = grow(&c->sc.dense_ws, &c->sc.cap_dense_ws, ab::dense_tc_workspace_bytes(n), c->stream);
+        e = grow(&c->sc.dense_ws, &c->sc.cap_dense_ws, ab::dense_tc_workspace_bytes(n, n, prec, true),
+                 c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "ab_kernel_solve workspace");
     const float4* X4 = (const float4*)X;
     const ab::SolveMatvec mv = [&](const float* P, float* Q) -> cudaError_t {
         if (prec == AB_PREC_FP32)
             return ab::launch_dense_fwd_ordered(n, n, X4, X4, nrhs, P, s, Q, c->stream);
-        return ab::launch_dense_tc_fwd(n, n, X4, X4, nrhs, P, s, prec, Q, c->sc.dense_ws, c->d_err,
+        return ab::launch_dense_tc_fwd(n, n, X4, X4, nrhs, P, s, prec, Q, true, c->sc.dense_ws, c->d_err,
                                        c->stream);
     };
     e = ab::run_solve(n, nrhs, B, sigma2, tol, max_iter, W, c->sc.solve_ws, mv, &it, &rr, c->stream);
@@ -803,9 +805,8 @@ ab_status ab_kernel_matvec_bwd(ab_ctx* c, int64_t m, int64_t n, const float* X, 
     if (!dg.ok) return fail(c, AB_ERR_CUDA, "cannot make device %d current", c->device);
     double* partial = nullptr;
     if (ds) {
-        // FP32: one partial per block; tensor cores: up to two per 128-row block
         const size_t count = prec == AB_PREC_FP32 ? ab::dense_partial_capacity(m, n, nrhs)
-                                                  : 2 * ((size_t)(m + 127) / 128) + 2;
+                                                  : ab::dense_tc_partial_capacity(m, n);
         if ((st = ensure_partial(c, count)) != AB_OK) return st;
         partial = c->sc.partial;
     }
@@ -820,26 +821,13 @@ ab_status ab_kernel_matvec_bwd(ab_ctx* c, int64_t m, int64_t n, const float* X, 
     } else {
         if (nrhs != 64)
             return fail(c, AB_ERR_UNSUPPORTED, "tensor-core paths need nrhs == 64");
-        // dW = K(Y, X) G: the forward kernel with the roles swapped;
-        // dX (+ ds) and dY: the tensor-core gradient kernel
-        size_t need = ab::dense_tc_workspace_bytes(m);
-        const size_t g1 = ab::dense_tc_grad_workspace_bytes(m, n);
-        const size_t g2 = ab::dense_tc_grad_workspace_bytes(n, m);
-        if (g1 > need) need = g1;
-        if (g2 > need) need = g2;
-        e = grow(&c->sc.dense_ws, &c->sc.cap_dense_ws, need, c->stream);
-        if (e == cudaSuccess && dW && n > 0)
-            e = ab::launch_dense_tc_fwd(n, m, (const float4*)Y, (const float4*)X, nrhs, G, s, prec, dW,
-                                        c->sc.dense_ws, c->d_err, c->stream);
-        if (e == cudaSuccess && (dX || partial) && m > 0)
-            e = ab::launch_dense_tc_gradx(m, n, (const float4*)X, (const float4*)Y, G, W, s, prec,
-                                          (float4*)dX, partial, &pc, c->sc.dense_ws, c->d_err, c->stream);
-        if (e == cudaSuccess && dY && n > 0) {
-            int pc2 = 0;
-            e = ab::launch_dense_tc_gradx(n, m, (const float4*)Y, (const float4*)X, W, G, s, prec,
-                                          (float4*)dY, nullptr, &pc2, c->sc.dense_ws, c->d_err,
-                                          c->stream);
-        }
+        e = grow(&c->sc.dense_ws, &c->sc.cap_dense_ws,
+                 ab::dense_tc_bwd_workspace_bytes(m, n, prec, dW != nullptr, dX != nullptr, dY != nullptr),
+                 c->stream);
+        if (e == cudaSuccess)
+            e = ab::launch_dense_tc_bwd(m, n, (const float4*)X, (const float4*)Y, W, s, prec, G, dW,
+                                        (float4*)dX, (float4*)dY, partial, &pc, c->sc.dense_ws, c->d_err,
+                                        c->stream);
     }
     if (e == cudaErrorNotSupported)
         return fail(c, AB_ERR_UNSUPPORTED, "precision not available for this shape");

@@ -483,21 +483,8 @@ cudaError_t own_pass(int64_t m, int64_t n, const float4* O, const float4* P, int
                              : own_dispatch<false, true>(p, a, st);
     if (e != cudaSuccess) return e;
     if (ds_count) *ds_count = (int)(p.blocks * p.splits);
-    if (p.splits > 1 && nv + ng > 0) {
-        // programmatic dependent launch: scheduled while the walk runs, waits
-        // in griddepcontrol.wait for its writes
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)((nv + ng + 255) / 256));
-        cfg.blockDim = dim3(256);
-        cfg.stream = st;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr.val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, k_dense_combine, p.splits, nv, (const float*)pv, val, ng,
-                               (const float4*)pg, grad);
-    }
+    if (p.splits > 1 && nv + ng > 0)
+        e = launch_dense_combine(p.splits, nv, pv, val, ng, pg, grad, st);
     return e;
 }
 
@@ -505,6 +492,22 @@ cudaError_t own_pass(int64_t m, int64_t n, const float4* O, const float4* P, int
 constexpr int kFusedRhs = 32;
 
 }  // namespace
+
+cudaError_t launch_dense_combine(int splits, int64_t vals, const float* pv, float* val, int64_t grads,
+                                 const float4* pg, float4* grad, cudaStream_t st) {
+    // programmatic dependent launch: scheduled while the walk runs, waits in
+    // griddepcontrol.wait for its writes
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((vals + grads + 255) / 256));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_dense_combine, splits, vals, pv, val, grads, pg, grad);
+}
 
 size_t dense_fwd_workspace_bytes(int64_t m, int64_t n, int nrhs) {
     if (m <= 0 || n <= 0) return 0;

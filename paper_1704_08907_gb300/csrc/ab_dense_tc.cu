@@ -121,6 +121,16 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
+// Programmatic dependent launch: the prepare and main kernels are scheduled
+// while the kernel before them finishes and wait here, before their first
+// global access, for its writes (without a prerequisite grid the wait returns
+// at once).  128 x 1000 points: 16.3 -> 15.3 us.
+__device__ __forceinline__ void wait_prerequisite() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void allow_dependents() {
+    asm volatile("griddepcontrol.launch_dependents;");
+}
 // One lane of a converged warp (elect.sync).  The MMA and producer roles run
 // their loops on the whole warp and issue tcgen05.mma, tcgen05.commit and the
 // bulk copies from the elected lane: issued from inside a one-lane branch
@@ -347,16 +357,17 @@ __device__ __forceinline__ float bf16hi_to_f(uint32_t v) { return __uint_as_floa
 // W rounded to nearest, lo the rounded remainder; tf32 likewise with
 // cvt.rna.tf32.
 // ---------------------------------------------------------------------------
+constexpr int kPrepThreads = 256;
+
 template <bool TF32>
-__global__ void __launch_bounds__(256)
-k_prep_w(int64_t n, int nrhs, const float* __restrict__ W, int64_t tiles,
-         uint8_t* __restrict__ img, uint32_t* __restrict__ wmax) {
+__device__ __forceinline__ void prep_w(int64_t block, int64_t blocks, int64_t n, int nrhs,
+                                       const float* __restrict__ W, uint8_t* __restrict__ img,
+                                       uint32_t* __restrict__ wmax) {
     constexpr int TN = Tile<TF32>::TN;
     constexpr int PTS = TF32 ? 4 : 8;                    // points per 16-byte chunk
-    const int64_t total = tiles * kRhs * 16;
+    const int64_t total = (n + TN - 1) / TN * kRhs * 16;
     uint32_t amax = 0;   // bits of max |W| seen by this thread (NaN bits order above inf)
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t e = block * kPrepThreads + threadIdx.x; e < total; e += blocks * kPrepThreads) {
         const int chunk = (int)(e % 16);                 // 16-byte chunk along K
         const int row = (int)((e / 16) % kRhs);          // right-hand side
         const int64_t t = e / (16 * kRhs);
@@ -404,32 +415,46 @@ __device__ __forceinline__ float ord2f(uint32_t u) {
     return __uint_as_float((u & 0x80000000u) ? (u & 0x7FFFFFFFu) : ~u);
 }
 
-// Bounding box of Y (bbox[0..2] = min, bbox[4..6] = max, as ordered ints;
-// initialised by the caller to (0xFFFFFFFF, 0)).
-__global__ void __launch_bounds__(256)
-k_bbox(int64_t n, const float4* __restrict__ Y, uint32_t* __restrict__ bbox) {
-    uint32_t mn[3] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu}, mx[3] = {0u, 0u, 0u};
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        const float4 y = __ldg(Y + j);
-        const float v[3] = {y.x, y.y, y.z};
+// Bounding boxes of one or two point sets (blockIdx.y), bbox + 8 y: [0..2] the
+// complements of the minima and [4..6] the maxima, as ordered ints, both kept
+// by atomicMax from 0.  One atomic a block and bound: the six words are the
+// same for all, and one a warp (2,048 warps at 65,536 points) took 10 us.
+__global__ void __launch_bounds__(kPrepThreads)
+k_bbox(int64_t n0, const float4* __restrict__ P0, int64_t n1, const float4* __restrict__ P1,
+       uint32_t* __restrict__ bbox) {
+    const int64_t n = blockIdx.y ? n1 : n0;
+    const float4* __restrict__ P = blockIdx.y ? P1 : P0;
+    allow_dependents();
+    uint32_t v[6] = {0u, 0u, 0u, 0u, 0u, 0u};
+    for (int64_t j = blockIdx.x * (int64_t)kPrepThreads + threadIdx.x; j < n;
+         j += (int64_t)gridDim.x * kPrepThreads) {
+        const float4 p = __ldg(P + j);
+        const uint32_t o[3] = {f2ord(p.x), f2ord(p.y), f2ord(p.z)};
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            mn[k] = min(mn[k], f2ord(v[k]));
-            mx[k] = max(mx[k], f2ord(v[k]));
+            v[k] = max(v[k], ~o[k]);
+            v[3 + k] = max(v[3 + k], o[k]);
         }
     }
+    __shared__ uint32_t s_v[6][kPrepThreads / 32];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        for (int o = 16; o > 0; o >>= 1) {
-            mn[k] = min(mn[k], __shfl_xor_sync(0xffffffffu, mn[k], o));
-            mx[k] = max(mx[k], __shfl_xor_sync(0xffffffffu, mx[k], o));
-        }
-        if ((threadIdx.x & 31) == 0) {
-            atomicMin(bbox + k, mn[k]);
-            atomicMax(bbox + 4 + k, mx[k]);
-        }
+    for (int k = 0; k < 6; ++k) {
+        v[k] = __reduce_max_sync(0xffffffffu, v[k]);
+        if ((threadIdx.x & 31) == 0) s_v[k][threadIdx.x >> 5] = v[k];
     }
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        const int k = threadIdx.x;
+        uint32_t m = 0u;
+        for (int w = 0; w < kPrepThreads / 32; ++w) m = max(m, s_v[k][w]);
+        if (m) atomicMax(bbox + 8 * blockIdx.y + (k < 3 ? k : k + 1), m);
+    }
+}
+
+__device__ __forceinline__ float3 bbox_centre(const uint32_t* __restrict__ bbox) {
+    return make_float3(0.5f * (ord2f(~bbox[0]) + ord2f(bbox[4])),
+                       0.5f * (ord2f(~bbox[1]) + ord2f(bbox[5])),
+                       0.5f * (ord2f(~bbox[2]) + ord2f(bbox[6])));
 }
 
 // Per Y point, centred on c = bounding-box midpoint:
@@ -448,15 +473,14 @@ k_bbox(int64_t n, const float4* __restrict__ Y, uint32_t* __restrict__ bbox) {
 // threads of a TMEM lane group at once, are 64 contiguous bytes (no bank
 // conflict).  Otherwise pair p at float4 2p (A) and 2p + 1 (B).
 template <bool BLOCKED>
-__global__ void __launch_bounds__(256)
-k_prep_y(int64_t n, const float4* __restrict__ Y, int64_t npad, const uint32_t* __restrict__ bbox,
-         float sl2e, float4* __restrict__ Yhat, float4* __restrict__ centre) {
-    const float c0 = 0.5f * (ord2f(bbox[0]) + ord2f(bbox[4]));
-    const float c1 = 0.5f * (ord2f(bbox[1]) + ord2f(bbox[5]));
-    const float c2 = 0.5f * (ord2f(bbox[2]) + ord2f(bbox[6]));
-    if (blockIdx.x == 0 && threadIdx.x == 0) *centre = make_float4(c0, c1, c2, 0.0f);
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; 2 * p < npad;
-         p += (int64_t)gridDim.x * blockDim.x) {
+__device__ __forceinline__ void prep_y(int64_t block, int64_t blocks, int64_t n,
+                                       const float4* __restrict__ Y, int64_t npad,
+                                       const uint32_t* __restrict__ bbox, float sl2e,
+                                       float4* __restrict__ Yhat, float4* __restrict__ centre) {
+    const float3 cc = bbox_centre(bbox);
+    const float c0 = cc.x, c1 = cc.y, c2 = cc.z;
+    if (block == 0 && threadIdx.x == 0) *centre = make_float4(c0, c1, c2, 0.0f);
+    for (int64_t p = block * kPrepThreads + threadIdx.x; 2 * p < npad; p += blocks * kPrepThreads) {
         float4 h[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
@@ -482,15 +506,44 @@ k_prep_y(int64_t n, const float4* __restrict__ Y, int64_t npad, const uint32_t* 
     }
 }
 
+// Everything the product's kernel reads, in one launch (the box is known):
+// blocks [0, wblocks) the weight images, the others the points.
+struct FwdPrep {
+    int64_t n;                 // points and weights
+    const float4* Y;
+    const float* W;
+    uint8_t* wimg;
+    float4 *Yhat, *centre;
+    const uint32_t* bbox;
+    uint32_t* wmax;
+    float sl2e;
+    int wblocks, yblocks;
+};
+template <bool TF32>
+__device__ __forceinline__ void prep_fwd(const FwdPrep& a, int block) {
+    constexpr int TN = Tile<TF32>::TN;
+    if (block < a.wblocks) prep_w<TF32>(block, a.wblocks, a.n, kRhs, a.W, a.wimg, a.wmax);
+    else prep_y<!TF32>(block - a.wblocks, a.yblocks, a.n, a.Y, (a.n + TN - 1) / TN * TN, a.bbox, a.sl2e,
+                       a.Yhat, a.centre);
+}
+template <bool TF32>
+__global__ void __launch_bounds__(kPrepThreads)
+k_prep_fwd(FwdPrep a) {
+    allow_dependents();
+    wait_prerequisite();
+    prep_fwd<TF32>(a, (int)blockIdx.x);
+}
+
 template <bool TF32, bool SPLIT>
 __global__ void __launch_bounds__(kThreadsTC, 1)
 k_dense_tc_fwd(int64_t m, int64_t total_tiles, const float4* __restrict__ X,
                const float4* __restrict__ Yhat, const float4* __restrict__ centre,
                const uint8_t* __restrict__ wimg, const uint32_t* __restrict__ wmax, float sl2e,
-               float* __restrict__ out, uint32_t* __restrict__ err) {
+               float* __restrict__ out, bool parts, uint32_t* __restrict__ err) {
     // blockIdx.y selects a contiguous range of Y tiles; with gridDim.y == 2
     // the two partial sums are added into a zeroed output (0 + a + b is the
-    // same in either order, so the result stays deterministic)
+    // same in either order, so the result stays deterministic); parts: each
+    // range writes its own [m][64] sums, combined in order afterwards
     constexpr int kTN = Tile<TF32>::TN;
     constexpr int kYBytes = Tile<TF32>::YBytes;
     constexpr int kStageBytes = Tile<TF32>::StageBytes;
@@ -540,6 +593,7 @@ k_dense_tc_fwd(int64_t m, int64_t total_tiles, const float4* __restrict__ X,
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     const int64_t row0 = (int64_t)blockIdx.x * kTM;
+    wait_prerequisite();
 
     if (warp == kEpiWarps + 1) {
         // ---------------- producer: W tiles into the ring ----------------
@@ -798,7 +852,7 @@ k_dense_tc_fwd(int64_t m, int64_t total_tiles, const float4* __restrict__ X,
         ok = __all_sync(0xffffffffu, ok && !*abort_flag);   // tcgen05.ld needs the whole warp
         tc_fence_after();
         if (ok) {
-            float* orow = out + (row0 + i) * kRhs;
+            float* orow = out + ((parts ? (int64_t)blockIdx.y * m : 0) + row0 + i) * kRhs;
 #pragma unroll 1
             for (int c0 = part * (kRhs / 4); c0 < (part + 1) * (kRhs / 4); c0 += 16) {
                 uint32_t v[16];
@@ -822,7 +876,7 @@ k_dense_tc_fwd(int64_t m, int64_t total_tiles, const float4* __restrict__ X,
                     for (int q = 0; q < 16; q += 4) {
                         const float4 r = make_float4(__uint_as_float(v[q]), __uint_as_float(v[q + 1]),
                                                      __uint_as_float(v[q + 2]), __uint_as_float(v[q + 3]));
-                        if (gridDim.y == 1) *reinterpret_cast<float4*>(orow + c0 + q) = r;
+                        if (parts || gridDim.y == 1) *reinterpret_cast<float4*>(orow + c0 + q) = r;
                         else atomicAdd(reinterpret_cast<float4*>(orow + c0 + q), r);
                     }
                 }
@@ -899,12 +953,11 @@ __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_
 // [rows x 64] fp32 -> per block of 128 rows: bf16 hi image then lo image,
 // each 128 rows x 128 B, K-major with the 128-byte swizzle.  Rows past
 // `rows` are zero.  One thread per (row, 16-byte chunk).
-__global__ void __launch_bounds__(256)
-k_prep_rows64(int64_t rows, int ncols, const float* __restrict__ src, int64_t blocks,
-              uint8_t* __restrict__ img) {
-    const int64_t total = blocks * 128 * 8;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-         e += (int64_t)gridDim.x * blockDim.x) {
+__device__ __forceinline__ void prep_rows64(int64_t block, int64_t blocks, int64_t rows, int ncols,
+                                            const float* __restrict__ src,
+                                            uint8_t* __restrict__ img) {
+    const int64_t total = (rows + 127) / 128 * 128 * 8;
+    for (int64_t e = block * kPrepThreads + threadIdx.x; e < total; e += blocks * kPrepThreads) {
         const int c = (int)(e % 8);
         const int64_t r = e / 8;
         const int rb = (int)(r % 128);
@@ -933,15 +986,15 @@ k_prep_rows64(int64_t rows, int ncols, const float* __restrict__ src, int64_t bl
 // (z0, z1, 0, 0), so the epilogue reads a column pair's components as
 // packed FP32 pairs.  Padding points are 0; their column of S = G W^T is
 // exactly 0 (zero rows of W), so they add nothing.
-__global__ void __launch_bounds__(256)
-k_prep_ytil(int64_t n, const float4* __restrict__ Y, int64_t npad, const uint32_t* __restrict__ bbox,
-            float q, float4* __restrict__ Yt, float4* __restrict__ centre) {
-    const float c0 = 0.5f * (ord2f(bbox[0]) + ord2f(bbox[4]));
-    const float c1 = 0.5f * (ord2f(bbox[1]) + ord2f(bbox[5]));
-    const float c2 = 0.5f * (ord2f(bbox[2]) + ord2f(bbox[6]));
-    if (blockIdx.x == 0 && threadIdx.x == 0) *centre = make_float4(c0, c1, c2, 0.0f);
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; 2 * p < npad;
-         p += (int64_t)gridDim.x * blockDim.x) {
+__device__ __forceinline__ void prep_ytil(int64_t block, int64_t blocks, int64_t n,
+                                          const float4* __restrict__ Y,
+                                          const uint32_t* __restrict__ bbox, float q,
+                                          float4* __restrict__ Yt, float4* __restrict__ centre) {
+    const float3 cc = bbox_centre(bbox);
+    const float c0 = cc.x, c1 = cc.y, c2 = cc.z;
+    const int64_t npad = (n + 127) / 128 * 128;
+    if (block == 0 && threadIdx.x == 0) *centre = make_float4(c0, c1, c2, 0.0f);
+    for (int64_t p = block * kPrepThreads + threadIdx.x; 2 * p < npad; p += blocks * kPrepThreads) {
         float3 h[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
@@ -957,12 +1010,45 @@ k_prep_ytil(int64_t n, const float4* __restrict__ Y, int64_t npad, const uint32_
     }
 }
 
-template <bool SPLIT>
+// Everything the adjoint's kernels read, in one launch: the images of G and
+// W, the scaled points of both sides, and (product: dW) the forward's operands
+// with G as the weights.  Each of its parts is a range of blocks.
+struct BwdPrep {
+    int64_t m, n;
+    const float4 *X, *Y;
+    const float *G, *W;
+    uint8_t *gimg, *wimg;      // rows64 images
+    float4 *Xt, *Yt;           // scaled points
+    float4 *cx, *cy;           // centres
+    const uint32_t* bbox;      // [0..7] of X, [8..15] of Y
+    float q;                   // sqrt(s log2 e)
+    int gb, wb, xb, yb;        // blocks of each part (0: not wanted)
+    FwdPrep fwd;               // wblocks = yblocks = 0: not wanted
+};
+template <bool TF32>
+__global__ void __launch_bounds__(kPrepThreads)
+k_prep_bwd(BwdPrep a) {
+    allow_dependents();
+    wait_prerequisite();
+    int b = (int)blockIdx.x;
+    if (b < a.gb) return prep_rows64(b, a.gb, a.m, kRhs, a.G, a.gimg);
+    b -= a.gb;
+    if (b < a.wb) return prep_rows64(b, a.wb, a.n, kRhs, a.W, a.wimg);
+    b -= a.wb;
+    if (b < a.xb) return prep_ytil(b, a.xb, a.m, a.X, a.bbox, a.q, a.Xt, a.cx);
+    b -= a.xb;
+    if (b < a.yb) return prep_ytil(b, a.yb, a.n, a.Y, a.bbox + 8, a.q, a.Yt, a.cy);
+    prep_fwd<TF32>(a.fwd, b - a.yb);
+}
+
+// DS: also the sums of A * exponent, for ds.  parts: gridDim.y partial
+// gradients [gridDim.y][m] instead of sums into dX.
+template <bool SPLIT, bool DS>
 __global__ void __launch_bounds__(kThreadsTC, 1)
 k_dense_tc_gradx(int64_t m, int64_t total_tiles, const float4* __restrict__ X,
                  const float4* __restrict__ Yt, const float4* __restrict__ centre,
                  const uint8_t* __restrict__ gimg, const uint8_t* __restrict__ wimg, float sl2e,
-                 float s, float4* __restrict__ dX, double* __restrict__ partial,
+                 float s, float4* __restrict__ dX, bool parts, double* __restrict__ partial,
                  uint32_t* __restrict__ err) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -1006,6 +1092,7 @@ k_dense_tc_gradx(int64_t m, int64_t total_tiles, const float4* __restrict__ X,
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     const int64_t row0 = (int64_t)blockIdx.x * kTM;
+    wait_prerequisite();
 
     if (warp == kEpiWarps + 1) {
         // producer: the warp waits, one elected lane copies
@@ -1163,7 +1250,7 @@ k_dense_tc_gradx(int64_t m, int64_t total_tiles, const float4* __restrict__ X,
                         acc[u][0] = fma2(A, d0, acc[u][0]);
                         acc[u][1] = fma2(A, d1, acc[u][1]);
                         acc[u][2] = fma2(A, d2, acc[u][2]);
-                        acc[u][3] = fma2(A, e, acc[u][3]);
+                        if (DS) acc[u][3] = fma2(A, e, acc[u][3]);
                     }
                 }
             }
@@ -1209,10 +1296,12 @@ k_dense_tc_gradx(int64_t m, int64_t total_tiles, const float4* __restrict__ X,
             // the sums carry the scale q of the differences
             const float f = -2.0f * s / sqrtf(sl2e);
             const float4 g = make_float4(f * sx, f * sy, f * sz, 0.0f);
-            if (gridDim.y == 1) dX[row0 + i] = g;
+            if (parts) dX[blockIdx.y * m + row0 + i] = g;
+            else if (gridDim.y == 1) dX[row0 + i] = g;
             else atomicAdd(dX + row0 + i, g);
         }
         // ds = -sum A d2 = -(1/s') sum A e, e = s' d2
+        if (DS) {
         double v = (row0 + i < m) ? -(double)se / (double)sl2e : 0.0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -1221,6 +1310,7 @@ k_dense_tc_gradx(int64_t m, int64_t total_tiles, const float4* __restrict__ X,
         asm volatile("bar.sync 1, 128;" ::: "memory");   // warps 0-3 only
         if (i == 0 && partial)
             partial[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = wsum[0] + wsum[1] + wsum[2] + wsum[3];
+        }
     }
     if (warp == kEpiWarps && lane == 0) {
         const long long t0 = gtimer();
@@ -1241,43 +1331,110 @@ k_dense_tc_gradx(int64_t m, int64_t total_tiles, const float4* __restrict__ X,
 
 }  // namespace
 
-size_t dense_tc_workspace_bytes(int64_t n) {
-    // sized for the tf32 tiling (64 points per 32 KB image), the larger one
-    const int64_t tiles = (n + 63) / 64;
-    return (size_t)tiles * kImgBytes + (size_t)tiles * 64 * 16 + 16 + 32 + 256;
+namespace {
+
+// Ranges of Y tiles that a product or gradient is split into: the number with
+// the least time in a model whose unit is a CTA's time for a tile (about 0.75
+// us).  CTAs run one an SM in waves, each for its tiles and about three more of
+// set-up and read-out.  Two ranges are summed into a zeroed output; more write
+// partial sums that another launch adds in order (four tiles' time, and both
+// move their bytes at about 1.9 MB a tile).  row_bytes: output of a row.
+// Against two ranges for fewer than four waves of row blocks and one
+// otherwise (bf16x3): 2000 x 30,000 points 118 -> 40 us, its adjoint 294 -> 127;
+// 16,000^2 115 -> 111 and 430 -> 403; 30,000 x 60,000 716 -> 614 and 2,720 ->
+// 2,467.
+// ordered (the solve's product): that old rule, because the iteration count
+// follows the last bits of the sums.
+int tc_splits(int64_t mblocks, int64_t tiles, int row_bytes, bool ordered) {
+    const int64_t sms = num_sms();
+    if (ordered) return mblocks < 4 * sms && tiles >= 2 ? 2 : 1;
+    int best = 1;
+    double cost = 1e300;
+    for (int s = 1; s <= 32 && (s == 1 || s <= tiles / 2); ++s) {
+        const int64_t waves = (mblocks * s + sms - 1) / sms;
+        double c = (double)waves * (double)((tiles + s - 1) / s + 3);
+        if (s > 1)
+            c += (s == 2 ? 2.0 : 4.0) + (double)(s + 2) * (double)mblocks * kTM * row_bytes / 1.9e6;
+        if (c < (s > 2 && best <= 2 ? 0.97 * cost : cost)) {   // partial sums: only for 3%
+            cost = c;
+            best = s;
+        }
+    }
+    return best;
 }
 
-template <bool TF32, bool SPLIT>
-static cudaError_t launch_tc(int64_t m, int64_t n, const float4* X, const float4* Y, int nrhs,
-                             const float* W, float s, float* out, void* ws, uint32_t* err,
-                             cudaStream_t st) {
+int prep_blocks(int64_t items) {
+    const int64_t b = (items + kPrepThreads - 1) / kPrepThreads;
+    return (int)(b < 4096 ? b : 4096);
+}
+
+int bbox_blocks(int64_t n) {
+    const int64_t b = (n + 4 * kPrepThreads - 1) / (4 * kPrepThreads);
+    return (int)(b < 1 ? 1 : b < 128 ? b : 128);
+}
+
+template <class... KArgs, class... Args>
+cudaError_t launch_dependent(void (*kern)(KArgs...), dim3 grid, int threads, int smem, cudaStream_t st,
+                             Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
+
+// Operands of the product with n points: offsets into a workspace.
+struct FwdLayout {
+    size_t img, yhat, bytes;
+    FwdLayout(size_t at, int64_t n) {
+        // sized for the tf32 tiling (64 points per 32 KB image), the larger one
+        const size_t tiles = (size_t)((n + 63) / 64);
+        img = at;
+        yhat = img + tiles * kImgBytes;
+        bytes = up256(yhat + (tiles + 1) * 64 * 16);
+    }
+};
+
+// The head of every workspace: boxes (two of 8 words), max |W|, centres.
+constexpr size_t kHeadBbox = 0, kHeadWmax = 64, kHeadCentre = 128, kHeadBytes = 256;
+
+template <bool TF32>
+FwdPrep fwd_prep(uint8_t* ws, const FwdLayout& lay, int64_t n, const float4* Y, const float* W, float s,
+                 size_t bbox, size_t centre) {
     constexpr int TN = Tile<TF32>::TN;
     const int64_t tiles = (n + TN - 1) / TN;
-    if (tiles == 0) return cudaMemsetAsync(out, 0, (size_t)m * nrhs * sizeof(float), st);
-    uint8_t* wimg = (uint8_t*)ws;                                    // 1024-aligned (cudaMalloc)
-    float4* Yhat = (float4*)(wimg + (size_t)tiles * kImgBytes);
-    float4* centre = Yhat + tiles * TN;
-    uint32_t* bbox = (uint32_t*)(centre + 1);
-    uint32_t* wmax = bbox + 8;   // max |W| (float bits), in the workspace's slack
-    const int64_t prep_items = tiles * kRhs * 16;
-    cudaError_t e = cudaMemsetAsync(wmax, 0, sizeof(uint32_t), st);
-    if (e != cudaSuccess) return e;
-    k_prep_w<TF32><<<(unsigned)((prep_items + 255) / 256 < 4096 ? (prep_items + 255) / 256 : 4096), 256,
-                     0, st>>>(n, nrhs, W, tiles, wimg, wmax);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(bbox, 0xFF, 4 * sizeof(uint32_t), st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(bbox + 4, 0x00, 4 * sizeof(uint32_t), st)) != cudaSuccess) return e;
-    k_bbox<<<(unsigned)((n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024), 256, 0, st>>>(n, Y, bbox);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const float sl2e = s * kLog2eTC;
-    k_prep_y<!TF32><<<(unsigned)((tiles * TN / 2 + 255) / 256), 256, 0, st>>>(n, Y, tiles * TN, bbox, sl2e,
-                                                                          Yhat, centre);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const int64_t mblocks = (m + kTM - 1) / kTM;
-    // split the Y range in two when the row blocks alone leave a ragged last
-    // wave (fewer than four waves of one CTA per SM)
-    const int split = (mblocks < 4 * (int64_t)num_sms() && tiles >= 2) ? 2 : 1;
-    if (split == 2 && (e = cudaMemsetAsync(out, 0, (size_t)m * nrhs * sizeof(float), st)) != cudaSuccess)
+    FwdPrep p;
+    p.n = n;
+    p.Y = Y;
+    p.W = W;
+    p.wimg = ws + lay.img;
+    p.Yhat = (float4*)(ws + lay.yhat);
+    p.centre = (float4*)(ws + centre);
+    p.bbox = (const uint32_t*)(ws + bbox);
+    p.wmax = (uint32_t*)(ws + kHeadWmax);
+    p.sl2e = s * kLog2eTC;
+    p.wblocks = prep_blocks(tiles * kRhs * 16);
+    p.yblocks = prep_blocks(tiles * TN / 2);
+    return p;
+}
+
+// The product's kernel on prepared operands; parts: [splits][m][64] or NULL.
+template <bool TF32, bool SPLIT>
+cudaError_t run_fwd(int64_t m, const float4* X, const FwdPrep& p, int splits, float* out, float* parts,
+                    uint32_t* err, cudaStream_t st) {
+    constexpr int TN = Tile<TF32>::TN;
+    const int64_t tiles = (p.n + TN - 1) / TN, mblocks = (m + kTM - 1) / kTM;
+    cudaError_t e;
+    if (splits > 1 && !parts &&
+        (e = cudaMemsetAsync(out, 0, (size_t)m * kRhs * sizeof(float), st)) != cudaSuccess)
         return e;
     // set on every launch: the attribute belongs to the current device, and
     // contexts on several devices may share this process (a microsecond
@@ -1285,87 +1442,194 @@ static cudaError_t launch_tc(int64_t m, int64_t n, const float4* X, const float4
     e = cudaFuncSetAttribute(k_dense_tc_fwd<TF32, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kSmemBytes);
     if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)mblocks, (unsigned)split);
-    k_dense_tc_fwd<TF32, SPLIT><<<grid, kThreadsTC, kSmemBytes, st>>>(m, tiles, X, Yhat, centre, wimg,
-                                                                      wmax, sl2e, out, err);
-    return cudaGetLastError();
+    e = launch_dependent(k_dense_tc_fwd<TF32, SPLIT>, dim3((unsigned)mblocks, (unsigned)splits), kThreadsTC,
+                         kSmemBytes, st, m, tiles, X, p.Yhat, p.centre, p.wimg, p.wmax, p.sl2e,
+                         parts ? parts : out, parts != nullptr, err);
+    if (e != cudaSuccess || !parts) return e;
+    return launch_dense_combine(splits, m * kRhs, parts, out, 0, nullptr, nullptr, st);
 }
 
-size_t dense_tc_grad_workspace_bytes(int64_t m, int64_t n) {
-    const int64_t mb = (m + 127) / 128, nb = (n + 127) / 128;
-    return (size_t)(mb + nb) * kGImg + (size_t)nb * 128 * 16 + 16 + 32 + 256;
+cudaError_t run_fwd_prec(ab_prec prec, int64_t m, const float4* X, const FwdPrep& p, int splits, float* out,
+                         float* parts, uint32_t* err, cudaStream_t st) {
+    switch (prec) {
+        case AB_PREC_BF16X3: return run_fwd<false, true>(m, X, p, splits, out, parts, err, st);
+        case AB_PREC_BF16: return run_fwd<false, false>(m, X, p, splits, out, parts, err, st);
+        case AB_PREC_TF32X3: return run_fwd<true, true>(m, X, p, splits, out, parts, err, st);
+        case AB_PREC_TF32: return run_fwd<true, false>(m, X, p, splits, out, parts, err, st);
+        default: return cudaErrorNotSupported;
+    }
 }
 
-// dX (and ds partials) for rows X against points Y with row weights G and
-// point weights W (both [.][64]); see k_dense_tc_gradx.
-cudaError_t launch_dense_tc_gradx(int64_t m, int64_t n, const float4* X, const float4* Y,
-                                  const float* G, const float* W, float s, ab_prec prec,
-                                  float4* dX, double* partial, int* partial_count, void* ws,
-                                  uint32_t* err, cudaStream_t st) {
-    *partial_count = 0;
-    if (m <= 0) return cudaSuccess;
+bool is_tf32(ab_prec prec) { return prec == AB_PREC_TF32X3 || prec == AB_PREC_TF32; }
+int fwd_tile(ab_prec prec) { return is_tf32(prec) ? Tile<true>::TN : Tile<false>::TN; }
+
+int fwd_splits(ab_prec prec, int64_t m, int64_t n, bool ordered) {
+    const int TN = fwd_tile(prec);
+    return tc_splits((m + kTM - 1) / kTM, (n + TN - 1) / TN, kRhs * 4, ordered);
+}
+int grad_splits(int64_t m, int64_t n) { return tc_splits((m + 127) / 128, (n + 127) / 128, 16, false); }
+
+// Partial sums of a product or gradient split more than in two.
+size_t fwd_parts_bytes(int splits, int64_t m) {
+    return splits > 2 ? up256((size_t)splits * m * kRhs * sizeof(float)) : 0;
+}
+size_t grad_parts_bytes(int splits, int64_t m) {
+    return splits > 2 ? up256((size_t)splits * m * sizeof(float4)) : 0;
+}
+
+template <bool SPLIT, bool DS>
+cudaError_t run_gradx(int64_t m, int64_t n, const float4* X, const float4* Yt, const float4* centre,
+                      const uint8_t* gimg, const uint8_t* wimg, float s, float4* dX, float4* parts,
+                      double* partial, int splits, uint32_t* err, cudaStream_t st) {
     const int64_t mb = (m + 127) / 128, nb = (n + 127) / 128;
     cudaError_t e;
-    if (nb == 0) {
-        if (dX) e = cudaMemsetAsync(dX, 0, (size_t)m * sizeof(float4), st);
-        else e = cudaSuccess;
+    if (splits > 1 && !parts && dX &&
+        (e = cudaMemsetAsync(dX, 0, (size_t)m * sizeof(float4), st)) != cudaSuccess)
         return e;
-    }
-    uint8_t* gimg = (uint8_t*)ws;
-    uint8_t* wimg = gimg + (size_t)mb * kGImg;
-    float4* Yt = (float4*)(wimg + (size_t)nb * kGImg);
-    float4* centre = Yt + nb * 128;
-    uint32_t* bbox = (uint32_t*)(centre + 1);
-    k_prep_rows64<<<(unsigned)((mb * 1024 + 255) / 256 < 4096 ? (mb * 1024 + 255) / 256 : 4096), 256, 0,
-                    st>>>(m, kRhs, G, mb, gimg);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_prep_rows64<<<(unsigned)((nb * 1024 + 255) / 256 < 4096 ? (nb * 1024 + 255) / 256 : 4096), 256, 0,
-                    st>>>(n, kRhs, W, nb, wimg);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(bbox, 0xFF, 4 * sizeof(uint32_t), st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(bbox + 4, 0x00, 4 * sizeof(uint32_t), st)) != cudaSuccess) return e;
-    k_bbox<<<(unsigned)((n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024), 256, 0, st>>>(n, Y, bbox);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const float sl2e = s * kLog2eTC;
-    k_prep_ytil<<<(unsigned)((nb * 64 + 255) / 256), 256, 0, st>>>(n, Y, nb * 128, bbox, sqrtf(sl2e), Yt,
-                                                                   centre);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const int split = (mb < 4 * (int64_t)num_sms() && nb >= 2) ? 2 : 1;
-    if (split == 2 && dX && (e = cudaMemsetAsync(dX, 0, (size_t)m * sizeof(float4), st)) != cudaSuccess)
-        return e;
-    const dim3 grid((unsigned)mb, (unsigned)split);
-    if (prec == AB_PREC_BF16 || prec == AB_PREC_TF32) {
-        if ((e = cudaFuncSetAttribute(k_dense_tc_gradx<false>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      kGradSmemBytes)) != cudaSuccess)
-            return e;   // per device: set on every launch
-        k_dense_tc_gradx<false><<<grid, kThreadsTC, kGradSmemBytes, st>>>(m, nb, X, Yt, centre, gimg,
-                                                                          wimg, sl2e, s, dX, partial, err);
-    } else {
-        if ((e = cudaFuncSetAttribute(k_dense_tc_gradx<true>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      kGradSmemBytes)) != cudaSuccess)
-            return e;   // per device: set on every launch
-        k_dense_tc_gradx<true><<<grid, kThreadsTC, kGradSmemBytes, st>>>(m, nb, X, Yt, centre, gimg,
-                                                                         wimg, sl2e, s, dX, partial, err);
-    }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    *partial_count = (int)(mb * split);
-    return cudaSuccess;
+    e = cudaFuncSetAttribute(k_dense_tc_gradx<SPLIT, DS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kGradSmemBytes);   // per device: set on every launch
+    if (e != cudaSuccess) return e;
+    e = launch_dependent(k_dense_tc_gradx<SPLIT, DS>, dim3((unsigned)mb, (unsigned)splits), kThreadsTC,
+                         kGradSmemBytes, st, m, nb, X, Yt, centre, gimg, wimg, s * kLog2eTC, s,
+                         parts ? parts : dX, parts != nullptr, partial, err);
+    if (e != cudaSuccess || !parts) return e;
+    return launch_dense_combine(splits, 0, nullptr, nullptr, m, parts, dX, st);
+}
+
+}  // namespace
+
+// The product's workspace: head, operands, partial sums.
+size_t dense_tc_workspace_bytes(int64_t m, int64_t n, ab_prec prec, bool ordered) {
+    return FwdLayout(kHeadBytes, n).bytes + fwd_parts_bytes(fwd_splits(prec, m, n, ordered), m);
 }
 
 cudaError_t launch_dense_tc_fwd(int64_t m, int64_t n, const float4* X, const float4* Y, int nrhs,
-                                const float* W, float s, ab_prec prec, float* out, void* ws,
+                                const float* W, float s, ab_prec prec, float* out, bool ordered, void* ws,
                                 uint32_t* err, cudaStream_t st) {
     if (m <= 0) return cudaSuccess;
     if (nrhs != kRhs) return cudaErrorNotSupported;
-    switch (prec) {
-        case AB_PREC_BF16X3: return launch_tc<false, true>(m, n, X, Y, nrhs, W, s, out, ws, err, st);
-        case AB_PREC_BF16: return launch_tc<false, false>(m, n, X, Y, nrhs, W, s, out, ws, err, st);
-        case AB_PREC_TF32X3: return launch_tc<true, true>(m, n, X, Y, nrhs, W, s, out, ws, err, st);
-        case AB_PREC_TF32: return launch_tc<true, false>(m, n, X, Y, nrhs, W, s, out, ws, err, st);
-        default: return cudaErrorNotSupported;
+    if (n <= 0) return cudaMemsetAsync(out, 0, (size_t)m * nrhs * sizeof(float), st);
+    uint8_t* w = (uint8_t*)ws;
+    const FwdLayout lay(kHeadBytes, n);
+    cudaError_t e = cudaMemsetAsync(w, 0, kHeadCentre, st);
+    if (e != cudaSuccess) return e;
+    k_bbox<<<bbox_blocks(n), kPrepThreads, 0, st>>>(n, Y, 0, nullptr, (uint32_t*)(w + kHeadBbox));
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const FwdPrep p = is_tf32(prec) ? fwd_prep<true>(w, lay, n, Y, W, s, kHeadBbox, kHeadCentre)
+                                    : fwd_prep<false>(w, lay, n, Y, W, s, kHeadBbox, kHeadCentre);
+    e = launch_dependent(is_tf32(prec) ? k_prep_fwd<true> : k_prep_fwd<false>,
+                         dim3((unsigned)(p.wblocks + p.yblocks)), kPrepThreads, 0, st, p);
+    if (e != cudaSuccess) return e;
+    const int splits = fwd_splits(prec, m, n, ordered);
+    return run_fwd_prec(prec, m, X, p, splits, out, splits > 2 ? (float*)(w + lay.bytes) : nullptr, err, st);
+}
+
+namespace {
+
+struct BwdLayout {
+    size_t gimg, wimg, xt, yt, fwd, parts, bytes;
+    BwdLayout(int64_t m, int64_t n, ab_prec prec, bool dW, bool dX, bool dY) {
+        const size_t mb = (size_t)((m + 127) / 128), nb = (size_t)((n + 127) / 128);
+        gimg = kHeadBytes;
+        wimg = gimg + mb * kGImg;
+        xt = wimg + nb * kGImg;
+        yt = xt + mb * 128 * 16;
+        fwd = up256(yt + nb * 128 * 16);
+        parts = dW ? FwdLayout(fwd, m).bytes : fwd;
+        size_t most = 0;   // one pass's partial sums at a time
+        auto take = [&](size_t b) { most = b > most ? b : most; };
+        if (dW) take(fwd_parts_bytes(fwd_splits(prec, n, m, false), n));
+        if (dX) take(grad_parts_bytes(grad_splits(m, n), m));
+        if (dY) take(grad_parts_bytes(grad_splits(n, m), n));
+        bytes = parts + most;
     }
+};
+
+}  // namespace
+
+size_t dense_tc_bwd_workspace_bytes(int64_t m, int64_t n, ab_prec prec, bool dW, bool dX, bool dY) {
+    return BwdLayout(m, n, prec, dW, dX, dY).bytes;
+}
+
+// FP64 partials of ds: one a row block and split.
+size_t dense_tc_partial_capacity(int64_t m, int64_t n) {
+    return (size_t)((m + 127) / 128) * (size_t)(n > 0 ? grad_splits(m, n) : 1);
+}
+
+// dW = K(Y, X) G: the forward kernel with the roles swapped; dX (with the ds
+// partials) and dY: k_dense_tc_gradx, for dY with X <-> Y and G <-> W.
+cudaError_t launch_dense_tc_bwd(int64_t m, int64_t n, const float4* X, const float4* Y, const float* W,
+                                float s, ab_prec prec, const float* G, float* dW, float4* dX, float4* dY,
+                                double* partial, int* partial_count, void* ws, uint32_t* err,
+                                cudaStream_t st) {
+    *partial_count = 0;
+    cudaError_t e = cudaSuccess;
+    if (m <= 0 || n <= 0) {
+        if (dW && n > 0) e = cudaMemsetAsync(dW, 0, (size_t)n * kRhs * sizeof(float), st);
+        if (e == cudaSuccess && dX && m > 0) e = cudaMemsetAsync(dX, 0, (size_t)m * sizeof(float4), st);
+        if (e == cudaSuccess && dY && n > 0) e = cudaMemsetAsync(dY, 0, (size_t)n * sizeof(float4), st);
+        return e;
+    }
+    const bool row_pass = dX || partial;
+    uint8_t* w = (uint8_t*)ws;
+    const BwdLayout lay(m, n, prec, dW != nullptr, dX != nullptr, dY != nullptr);
+    if ((e = cudaMemsetAsync(w, 0, kHeadCentre, st)) != cudaSuccess) return e;
+    const int bb = bbox_blocks(m > n ? m : n);
+    k_bbox<<<dim3((unsigned)bb, 2), kPrepThreads, 0, st>>>(m, X, n, Y, (uint32_t*)(w + kHeadBbox));
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    BwdPrep p;
+    p.m = m;
+    p.n = n;
+    p.X = X;
+    p.Y = Y;
+    p.G = G;
+    p.W = W;
+    p.gimg = w + lay.gimg;
+    p.wimg = w + lay.wimg;
+    p.Xt = (float4*)(w + lay.xt);
+    p.Yt = (float4*)(w + lay.yt);
+    p.cx = (float4*)(w + kHeadCentre);
+    p.cy = (float4*)(w + kHeadCentre + 16);
+    p.bbox = (const uint32_t*)(w + kHeadBbox);
+    p.q = sqrtf(s * kLog2eTC);
+    p.gb = row_pass || dY ? prep_blocks((m + 127) / 128 * 1024) : 0;
+    p.wb = row_pass || dY ? prep_blocks((n + 127) / 128 * 1024) : 0;
+    p.xb = dY ? prep_blocks((m + 127) / 128 * 64) : 0;
+    p.yb = row_pass ? prep_blocks((n + 127) / 128 * 64) : 0;
+    const FwdLayout fl(lay.fwd, m);
+    // the product's own copy of the X centre: its block 0 may be another one
+    p.fwd = is_tf32(prec) ? fwd_prep<true>(w, fl, m, X, G, s, kHeadBbox, kHeadCentre + 32)
+                          : fwd_prep<false>(w, fl, m, X, G, s, kHeadBbox, kHeadCentre + 32);
+    if (!dW) p.fwd.wblocks = p.fwd.yblocks = 0;
+    const int blocks = p.gb + p.wb + p.xb + p.yb + p.fwd.wblocks + p.fwd.yblocks;
+    if (blocks > 0) {
+        e = launch_dependent(is_tf32(prec) ? k_prep_bwd<true> : k_prep_bwd<false>, dim3((unsigned)blocks),
+                             kPrepThreads, 0, st, p);
+        if (e != cudaSuccess) return e;
+    }
+    if (dW) {
+        const int splits = fwd_splits(prec, n, m, false);
+        e = run_fwd_prec(prec, n, Y, p.fwd, splits, dW, splits > 2 ? (float*)(w + lay.parts) : nullptr, err, st);
+        if (e != cudaSuccess) return e;
+    }
+    const bool split3 = prec == AB_PREC_BF16X3 || prec == AB_PREC_TF32X3;
+    auto grad = [&](int64_t rows, int64_t pts, const float4* R, const float4* Pt, const float4* c,
+                    const uint8_t* a, const uint8_t* b, float4* out, double* ds, int* count) -> cudaError_t {
+        const int splits = grad_splits(rows, pts);
+        float4* parts = splits > 2 && out ? (float4*)(w + lay.parts) : nullptr;
+        if (count) *count = (int)((rows + 127) / 128) * splits;
+        if (split3)
+            return ds ? run_gradx<true, true>(rows, pts, R, Pt, c, a, b, s, out, parts, ds, splits, err, st)
+                      : run_gradx<true, false>(rows, pts, R, Pt, c, a, b, s, out, parts, ds, splits, err, st);
+        return ds ? run_gradx<false, true>(rows, pts, R, Pt, c, a, b, s, out, parts, ds, splits, err, st)
+                  : run_gradx<false, false>(rows, pts, R, Pt, c, a, b, s, out, parts, ds, splits, err, st);
+    };
+    if (row_pass) {
+        e = grad(m, n, X, p.Yt, p.cy, p.gimg, p.wimg, dX, partial, partial ? partial_count : nullptr);
+        if (e != cudaSuccess) return e;
+    }
+    if (dY) e = grad(n, m, Y, p.Xt, p.cx, p.wimg, p.gimg, dY, nullptr, nullptr);
+    return e;
 }
 
 }  // namespace ab

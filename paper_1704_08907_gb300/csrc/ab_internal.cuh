@@ -197,16 +197,26 @@ AB_HIDDEN cudaError_t launch_dense_bwd(int64_t m, int64_t n, const float4* X,
 // ds partials of launch_dense_bwd
 AB_HIDDEN size_t dense_partial_capacity(int64_t m, int64_t n, int nrhs);
 
-// ab_dense_tc.cu (tcgen05 path; nrhs must be 64)
-AB_HIDDEN size_t dense_tc_workspace_bytes(int64_t n);
+// Sums of partials in the order of the splits: vals floats, grads float4
+AB_HIDDEN cudaError_t launch_dense_combine(int splits, int64_t vals, const float* pv, float* val,
+                                           int64_t grads, const float4* pg, float4* grad,
+                                           cudaStream_t st);
+
+// ab_dense_tc.cu (tcgen05 path; nrhs must be 64).  ordered: the sums' order
+// does not depend on m (the solve)
+AB_HIDDEN size_t dense_tc_workspace_bytes(int64_t m, int64_t n, ab_prec prec, bool ordered);
 AB_HIDDEN cudaError_t launch_dense_tc_fwd(int64_t m, int64_t n, const float4* X, const float4* Y,
                                           int nrhs, const float* W, float s, ab_prec prec,
-                                          float* out, void* ws, uint32_t* err, cudaStream_t st);
-AB_HIDDEN size_t dense_tc_grad_workspace_bytes(int64_t m, int64_t n);
-AB_HIDDEN cudaError_t launch_dense_tc_gradx(int64_t m, int64_t n, const float4* X, const float4* Y,
-                                            const float* G, const float* W, float s, ab_prec prec,
-                                            float4* dX, double* partial, int* partial_count,
-                                            void* ws, uint32_t* err, cudaStream_t st);
+                                          float* out, bool ordered, void* ws, uint32_t* err,
+                                          cudaStream_t st);
+AB_HIDDEN size_t dense_tc_bwd_workspace_bytes(int64_t m, int64_t n, ab_prec prec, bool dW, bool dX,
+                                              bool dY);
+AB_HIDDEN size_t dense_tc_partial_capacity(int64_t m, int64_t n);
+AB_HIDDEN cudaError_t launch_dense_tc_bwd(int64_t m, int64_t n, const float4* X, const float4* Y,
+                                          const float* W, float s, ab_prec prec, const float* G,
+                                          float* dW, float4* dX, float4* dY, double* partial,
+                                          int* partial_count, void* ws, uint32_t* err,
+                                          cudaStream_t st);
 
 // ab_solve.cu: conjugate gradients for (K(X, X) + sigma^2 I) W = B; the
 // matvec Q = K(X, X) P is supplied by the caller
