@@ -452,9 +452,9 @@ k_bbox(int64_t n0, const float4* __restrict__ P0, int64_t n1, const float4* __re
 }
 
 __device__ __forceinline__ float3 bbox_centre(const uint32_t* __restrict__ bbox) {
-    return make_float3(0.5f * (ord2f(~bbox[0]) + ord2f(bbox[4])),
-                       0.5f * (ord2f(~bbox[1]) + ord2f(bbox[5])),
-                       0.5f * (ord2f(~bbox[2]) + ord2f(bbox[6])));
+    return make_float3(0.5f * (ord2f(~__ldcg(bbox)) + ord2f(__ldcg(bbox + 4))),
+                       0.5f * (ord2f(~__ldcg(bbox + 1)) + ord2f(__ldcg(bbox + 5))),
+                       0.5f * (ord2f(~__ldcg(bbox + 2)) + ord2f(__ldcg(bbox + 6))));
 }
 
 // Per Y point, centred on c = bounding-box midpoint:
@@ -690,7 +690,7 @@ k_dense_tc_fwd(int64_t m, int64_t total_tiles, const float4* __restrict__ X,
         // row in centred coordinates; a padding row gets -inf: K = 0
         float xa = 0.f, xb = 0.f, xc = 0.f, ci = -__int_as_float(0x7f800000);
         if (row0 + i < m) {
-            const float4 x = __ldg(X + row0 + i), c = __ldg(centre);
+            const float4 x = __ldg(X + row0 + i), c = __ldcg(centre);
             xa = x.x - c.x;
             xb = x.y - c.y;
             xc = x.z - c.z;
@@ -710,7 +710,7 @@ k_dense_tc_fwd(int64_t m, int64_t total_tiles, const float4* __restrict__ X,
             atomicMax(fm, __float_as_uint(row0 + i < m ? -ci : 0.0f));   // -ci >= 0 (or NaN)
             asm volatile("bar.sync 1, %0;" ::"r"(32 * kEpiWarps) : "memory");   // epilogue warps
             const float M = __uint_as_float(*(volatile uint32_t*)fm);
-            const float wm = __uint_as_float(__ldg(wmax));
+            const float wm = __uint_as_float(__ldcg(wmax));
             fold = M + log2f(wm) + log2f((float)total_tiles * Tile<TF32>::TN) < 120.0f;
         }
         // bf16 paths: thread (g4, c4) = (lane / 4, lane % 4) evaluates rows
@@ -719,7 +719,7 @@ k_dense_tc_fwd(int64_t m, int64_t total_tiles, const float4* __restrict__ X,
         const int g4 = lane >> 2, c4 = lane & 3;
         uint64_t xq[4][4];   // row r: xa, xb, xc, ci as duplicated pairs
         if (!TF32) {
-            const float4 c = __ldg(centre);
+            const float4 c = __ldcg(centre);
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 const int64_t row = row0 + quad * 32 + 8 * r + g4;
@@ -1193,7 +1193,7 @@ k_dense_tc_gradx(int64_t m, int64_t total_tiles, const float4* __restrict__ X,
         uint64_t xt[2][3];   // row u: x~ components as duplicated pairs (padding rows: S = 0)
         const float qs = sqrtf(sl2e);   // the scale of the y~ image
         {
-            const float4 c = __ldg(centre);
+            const float4 c = __ldcg(centre);
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 const int64_t row = row0 + quad * 32 + 16 * half + 8 * u + g4;

@@ -57,6 +57,14 @@ __device__ __forceinline__ void col_partial(double v, int c, int nrhs, double* p
     }
 }
 
+// The step kernels are programmatic dependent launches of the kernel before
+// them: scheduled while it finishes, they wait here for its writes, and read
+// what it wrote from L2.
+__device__ __forceinline__ void solve_dependent() {
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // R = B, P = B, W = 0; partial of b.b
 __global__ void __launch_bounds__(kCols * kRowLanes)
 k_solve_init(int64_t n, int nrhs, const float* __restrict__ B, float* __restrict__ R,
@@ -81,7 +89,9 @@ k_solve_init(int64_t n, int nrhs, const float* __restrict__ B, float* __restrict
 // partial of p.(q + sigma^2 p), q = K p
 __global__ void __launch_bounds__(kCols * kRowLanes)
 k_solve_pap(int64_t n, int nrhs, const float* __restrict__ P, const float* __restrict__ Q,
-            float sigma2, double* __restrict__ partial) {
+            float sigma2, double* __restrict__ partial, int* __restrict__ n_active) {
+    solve_dependent();
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0) *n_active = 0;
     const int c = blockIdx.y * kCols + threadIdx.x;
     int64_t r0, r1;
     row_range(n, r0, r1);
@@ -89,8 +99,8 @@ k_solve_pap(int64_t n, int nrhs, const float* __restrict__ P, const float* __res
     if (c < nrhs) {
         for (int64_t i = r0 + threadIdx.y; i < r1; i += kRowLanes) {
             const int64_t e = i * nrhs + c;
-            const double p = __ldg(P + e);
-            acc += p * ((double)__ldg(Q + e) + (double)sigma2 * p);
+            const double p = __ldcg(P + e);
+            acc += p * ((double)__ldcg(Q + e) + (double)sigma2 * p);
         }
     }
     col_partial(acc, c, nrhs, partial);
@@ -101,6 +111,7 @@ __global__ void __launch_bounds__(kCols * kRowLanes)
 k_solve_update(int64_t n, int nrhs, const float* __restrict__ P, const float* __restrict__ Q,
                float sigma2, const Col* __restrict__ col, float* __restrict__ R,
                float* __restrict__ W, double* __restrict__ partial) {
+    solve_dependent();
     const int c = blockIdx.y * kCols + threadIdx.x;
     int64_t r0, r1;
     row_range(n, r0, r1);
@@ -110,10 +121,10 @@ k_solve_update(int64_t n, int nrhs, const float* __restrict__ P, const float* __
         const float alpha = (k.active && k.pap > 0.0) ? (float)(k.rs / k.pap) : 0.0f;
         for (int64_t i = r0 + threadIdx.y; i < r1; i += kRowLanes) {
             const int64_t e = i * nrhs + c;
-            const float p = __ldg(P + e);
-            const float ap = fmaf(sigma2, p, __ldg(Q + e));
-            W[e] = fmaf(alpha, p, W[e]);
-            const float r = fmaf(-alpha, ap, R[e]);
+            const float p = __ldcg(P + e);
+            const float ap = fmaf(sigma2, p, __ldcg(Q + e));
+            W[e] = fmaf(alpha, p, __ldcg(W + e));
+            const float r = fmaf(-alpha, ap, __ldcg(R + e));
             R[e] = r;
             acc += (double)r * r;
         }
@@ -125,6 +136,7 @@ k_solve_update(int64_t n, int nrhs, const float* __restrict__ P, const float* __
 __global__ void __launch_bounds__(kCols * kRowLanes)
 k_solve_dir(int64_t n, int nrhs, const float* __restrict__ R, const Col* __restrict__ col,
             float* __restrict__ P) {
+    solve_dependent();
     const int c = blockIdx.y * kCols + threadIdx.x;
     int64_t r0, r1;
     row_range(n, r0, r1);
@@ -133,42 +145,47 @@ k_solve_dir(int64_t n, int nrhs, const float* __restrict__ R, const Col* __restr
     const float beta = (float)k.beta;
     for (int64_t i = r0 + threadIdx.y; i < r1; i += kRowLanes) {
         const int64_t e = i * nrhs + c;
-        P[e] = k.active ? fmaf(beta, P[e], __ldg(R + e)) : 0.0f;
+        P[e] = k.active ? fmaf(beta, __ldcg(P + e), __ldcg(R + e)) : 0.0f;
     }
 }
 
-// Column sums of the partials in a fixed order, then the scalar step for
-// what = 0: b.b (initialise), 1: p.Ap, 2: r'.r' (beta, activity, counts).
-__global__ void k_solve_finish(const double* __restrict__ partial, int blocks, int nrhs, int what,
-                               double tol2, Col* __restrict__ col, int* __restrict__ n_active) {
-    for (int c = threadIdx.x; c < nrhs; c += blockDim.x) {
-        double t = 0.0;
-        for (int b = 0; b < blocks; ++b) t += partial[(int64_t)b * nrhs + c];
-        Col k = col[c];
-        if (what == 0) {
-            k.bb = t;
+// Column sum of the partials in a fixed order, then the scalar step for
+// what = 0: b.b (initialise), 1: p.Ap, 2: r'.r' (beta, activity, counts).  One
+// warp and block a column: FP64 additions take an SM's pipe for 16 clocks and
+// more, and all columns on one SM took longer than the rest of a step.
+__global__ void __launch_bounds__(32)
+k_solve_finish(const double* __restrict__ partial, int blocks, int nrhs, int what, double tol2,
+               Col* __restrict__ col, int* __restrict__ n_active) {
+    solve_dependent();
+    const int c = blockIdx.x, lane = threadIdx.x;
+    double t = 0.0;
+    for (int b = lane; b < blocks; b += 32) t += __ldcg(partial + (int64_t)b * nrhs + c);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane != 0) return;
+    Col k = col[c];
+    if (what == 0) {
+        k.bb = t;
+        k.rs = t;
+        k.pap = 0.0;
+        k.rs_new = t;
+        k.beta = 0.0;
+        k.active = t > 0.0;
+    } else if (what == 1) {
+        k.pap = t;
+    } else {
+        k.rs_new = t;
+        if (k.active) {
+            k.beta = k.rs > 0.0 ? t / k.rs : 0.0;
             k.rs = t;
-            k.pap = 0.0;
-            k.rs_new = t;
-            k.beta = 0.0;
-            k.active = t > 0.0;
-        } else if (what == 1) {
-            k.pap = t;
+            k.active = t > tol2 * k.bb;
         } else {
-            k.rs_new = t;
-            if (k.active) {
-                k.beta = k.rs > 0.0 ? t / k.rs : 0.0;
-                k.rs = t;
-                k.active = t > tol2 * k.bb;
-            } else {
-                k.beta = 0.0;
-            }
+            k.beta = 0.0;
         }
-        col[c] = k;
-        if (what != 1 && k.active) atomicAdd(n_active, 1);
     }
+    col[c] = k;
+    if (what != 1 && k.active) atomicAdd(n_active, 1);
 }
-
 
 // ---------------------------------------------------------------------------
 // The whole iteration in one cooperative launch, for FP32 systems of few
@@ -596,9 +613,26 @@ k_solve_coop(CoopSolve a) {
     }
 }
 
+// Row blocks of the step kernels: 16 rows each (their FP64 sums are bound by
+// the FP64 pipes, so they want all SMs: 256 rows a block took 17-34 us a
+// kernel at n = 4096), at most 1024.
 int solve_blocks(int64_t n) {
-    const int64_t b = (n + 255) / 256;
+    const int64_t b = (n + 15) / 16;
     return (int)(b < 1024 ? (b > 0 ? b : 1) : 1024);
+}
+
+template <class... KArgs, class... Args>
+cudaError_t solve_launch(void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
 }  // namespace
@@ -717,11 +751,11 @@ cudaError_t run_solve(int64_t n, int nrhs, const float* B, float sigma2, float t
     int n_active = 0;
     cudaError_t e;
     auto finish = [&](int what) -> cudaError_t {
-        cudaError_t r = cudaMemsetAsync(n_active_dev, 0, sizeof(int), st);
-        if (r != cudaSuccess) return r;
-        k_solve_finish<<<1, 256, 0, st>>>(partial, blocks, nrhs, what, tol2, col, n_active_dev);
-        return cudaGetLastError();
+        return solve_launch(k_solve_finish, dim3((unsigned)nrhs), dim3(32), st, (const double*)partial, blocks,
+                            nrhs, what, tol2, col, n_active_dev);
     };
+    // the count of active columns starts each step at 0
+    if ((e = cudaMemsetAsync(n_active_dev, 0, sizeof(int), st)) != cudaSuccess) return e;
     k_solve_init<<<grid, block, 0, st>>>(n, nrhs, B, R, P, W, partial);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = finish(0)) != cudaSuccess) return e;
@@ -731,14 +765,14 @@ cudaError_t run_solve(int64_t n, int nrhs, const float* B, float sigma2, float t
     int it = 0;
     while (n_active > 0 && it < max_iter) {
         if ((e = mv(P, Q)) != cudaSuccess) return e;
-        k_solve_pap<<<grid, block, 0, st>>>(n, nrhs, P, Q, sigma2, partial);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if ((e = finish(1)) != cudaSuccess) return e;
-        k_solve_update<<<grid, block, 0, st>>>(n, nrhs, P, Q, sigma2, col, R, W, partial);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if ((e = finish(2)) != cudaSuccess) return e;
-        k_solve_dir<<<grid, block, 0, st>>>(n, nrhs, R, col, P);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = solve_launch(k_solve_pap, grid, block, st, n, nrhs, (const float*)P, (const float*)Q, sigma2,
+                         partial, n_active_dev);
+        if (e != cudaSuccess || (e = finish(1)) != cudaSuccess) return e;
+        e = solve_launch(k_solve_update, grid, block, st, n, nrhs, (const float*)P, (const float*)Q, sigma2,
+                         (const Col*)col, R, W, partial);
+        if (e != cudaSuccess || (e = finish(2)) != cudaSuccess) return e;
+        e = solve_launch(k_solve_dir, grid, block, st, n, nrhs, (const float*)R, (const Col*)col, P);
+        if (e != cudaSuccess) return e;
         ++it;
         if ((e = cudaMemcpyAsync(&n_active, n_active_dev, sizeof(int), cudaMemcpyDeviceToHost, st)) !=
             cudaSuccess)
