@@ -107,12 +107,19 @@ k_gather_w_pos(int64_t n, const uint32_t* __restrict__ perm, const float* __rest
         spos[s].w = __ldg(w + perm[s]);
 }
 
+// A pair of values a particle in sorted order: into sv, or in 2-D into the
+// third and fourth components of the sorted positions (the third is unused
+// there), where they come with the candidate's position.
+template <bool IN_POS>
 __global__ void __launch_bounds__(kThreads)
 k_gather_pairs(int64_t n, const uint32_t* __restrict__ perm, const float2* __restrict__ wv,
-               float2* __restrict__ sv) {
+               float2* __restrict__ sv, float4* __restrict__ spos) {
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n;
-         s += (int64_t)gridDim.x * blockDim.x)
-        sv[s] = __ldg(wv + perm[s]);
+         s += (int64_t)gridDim.x * blockDim.x) {
+        const float2 v = __ldg(wv + perm[s]);
+        if (IN_POS) reinterpret_cast<float2*>(spos + s)[1] = v;
+        else sv[s] = v;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1106,17 +1113,19 @@ cudaError_t launch_expand_cells(const CellList& cl, uint32_t* out, cudaStream_t 
     return cudaGetLastError();
 }
 
-// A per-particle scalar in sorted order: out[s] = v[perm[s]].
+// A per-particle scalar in sorted order: out[s * stride] = v[perm[s]].
 __global__ void __launch_bounds__(kThreads)
 k_gather_scalar(int64_t n, const uint32_t* __restrict__ perm, const float* __restrict__ v,
-                float* __restrict__ out) {
+                float* __restrict__ out, int stride) {
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n;
          s += (int64_t)gridDim.x * blockDim.x)
-        out[s] = __ldg(v + perm[s]);
+        out[s * stride] = __ldg(v + perm[s]);
 }
 
-// Two per-particle scalars in one pass over the permutation: g into the pad of
-// the sorted positions, w as out[s] = w[perm[s]].
+// The Gaussian adjoint's two scalars in one pass over the permutation: g into
+// the pad of the sorted positions, w into out[s], or (IN_POS, 2-D) into their
+// third component.
+template <bool IN_POS>
 __global__ void __launch_bounds__(kThreads)
 k_gather_pad_scalar(int64_t n, const uint32_t* __restrict__ perm, const float* __restrict__ g,
                     const float* __restrict__ w, float4* __restrict__ spos, float* __restrict__ out) {
@@ -1124,8 +1133,12 @@ k_gather_pad_scalar(int64_t n, const uint32_t* __restrict__ perm, const float* _
          s += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t p = perm[s];
         const float gs = __ldg(g + p), ws = __ldg(w + p);
-        spos[s].w = gs;
-        out[s] = ws;
+        if (IN_POS) {
+            reinterpret_cast<float2*>(spos + s)[1] = make_float2(ws, gs);
+        } else {
+            spos[s].w = gs;
+            out[s] = ws;
+        }
     }
 }
 
@@ -1136,11 +1149,14 @@ cudaError_t launch_gather_pad_scalar(const CellList& cl, const float* g, const f
     // at 16.7M points (2 x 67 MB) it took 400 us against 142 + 81 apart
     constexpr int64_t kOnePassMaxN = int64_t(1) << 22;
     const int grid = ew_grid(cl.n);
+    const bool in_pos = cl.g.dim == 2;
     if (cl.n <= kOnePassMaxN) {
-        k_gather_pad_scalar<<<grid, kThreads, 0, st>>>(cl.n, cl.perm, g, w, cl.spos, out);
+        if (in_pos) k_gather_pad_scalar<true><<<grid, kThreads, 0, st>>>(cl.n, cl.perm, g, w, cl.spos, out);
+        else k_gather_pad_scalar<false><<<grid, kThreads, 0, st>>>(cl.n, cl.perm, g, w, cl.spos, out);
     } else {
         k_gather_w_pos<<<grid, kThreads, 0, st>>>(cl.n, cl.perm, g, cl.spos);
-        k_gather_scalar<<<grid, kThreads, 0, st>>>(cl.n, cl.perm, w, out);
+        k_gather_scalar<<<grid, kThreads, 0, st>>>(cl.n, cl.perm, w, in_pos ? &cl.spos->z : out,
+                                                   in_pos ? 4 : 1);
     }
     return cudaGetLastError();
 }
@@ -1154,7 +1170,8 @@ cudaError_t launch_gather_w_pos(CellList& cl, const float* w, cudaStream_t st) {
 cudaError_t launch_gather_pairs(const CellList& cl, const float2* wv, float2* sv,
                                 cudaStream_t st) {
     if (cl.n <= 0) return cudaSuccess;
-    k_gather_pairs<<<ew_grid(cl.n), kThreads, 0, st>>>(cl.n, cl.perm, wv, sv);
+    if (cl.g.dim == 2) k_gather_pairs<true><<<ew_grid(cl.n), kThreads, 0, st>>>(cl.n, cl.perm, wv, sv, cl.spos);
+    else k_gather_pairs<false><<<ew_grid(cl.n), kThreads, 0, st>>>(cl.n, cl.perm, wv, sv, cl.spos);
     return cudaGetLastError();
 }
 

@@ -53,7 +53,7 @@ struct CellList {
     Geom g{};
     const float* user_pos = nullptr;  // caller's positions at build time
     bool valid = false;
-    float4* spos = nullptr;           // sorted positions (x, y, z, 0)
+    float4* spos = nullptr;           // sorted positions (x, y, z, value; 2-D: x, y, two values)
     uint32_t* perm = nullptr;         // perm[s] = original index
     uint2* cell_rank = nullptr;       // per original particle: (cell, atomic arrival rank)
     uint32_t* tmp = nullptr;          // unordered slot -> original index
@@ -125,10 +125,12 @@ AB_HIDDEN cudaError_t launch_build_radix(CellList& cl, const float* pos, bool pa
 // c = 0 .. n_cells (device uint32[n_cells + 1]).
 AB_HIDDEN cudaError_t launch_expand_cells(const CellList& cl, uint32_t* out, cudaStream_t st);
 AB_HIDDEN cudaError_t launch_gather_w_pos(CellList& cl, const float* w, cudaStream_t st);
-// g into the pad of the sorted positions and out[s] = w[perm[s]]
+// g into the pad of the sorted positions and out[s] = w[perm[s]] (2-D: w into
+// their z component)
 AB_HIDDEN cudaError_t launch_gather_pad_scalar(const CellList& cl, const float* g, const float* w,
                                                float* out, cudaStream_t st);
-// sv[s] = wv[perm[s]]: a per-particle pair of values into sorted order
+// sv[s] = wv[perm[s]]: a per-particle pair of values into sorted order (2-D:
+// into the z and pad components of the sorted positions)
 AB_HIDDEN cudaError_t launch_gather_pairs(const CellList& cl, const float2* wv, float2* sv,
                                           cudaStream_t st);
 // Exclusive scan of n u32 counts into out (u32 or u64), out[n] = total.

@@ -25,16 +25,15 @@ k_pair_fwd(PairParams P, PairOut o) {
                 a0 += 1.0f;
             } else if (OP == AB_OP_GAUSS) {
                 a0 = fmaf(pj.w, ex2_approx(-P.s_log2e * d2), a0);
-            } else {   // SPH_DENSITY: m_j W(d)
-                float q;
-                const float t = wend_t(d2, P.inv_r, q);
-                const float t2 = t * t;
-                a0 = fmaf(pj.w * P.wend_a, t2 * t2 * fmaf(4.0f, q, 1.0f), a0);
+            } else {   // SPH_DENSITY: m_j W(d) / a
+                // (1 - q)^4 (1 + 4 q), q = d / r, in t = 1 - q
+                const float t = fmaf(-P.inv_r, pair_distance(d2), 1.0f), t2 = t * t;
+                a0 = fmaf(pj.w, t2 * t2 * fmaf(-4.0f, t, 5.0f), a0);
             }
         });
     a0 = lane_sum<SL>(a0);
     if (SL > 0 && (!live || sub != 0)) return;
-    if (OP == AB_OP_SPH_DENSITY) a0 = fmaf(pi.w, P.wend_a, a0);   // the particle itself
+    if (OP == AB_OP_SPH_DENSITY) a0 = (a0 + pi.w) * P.wend_a;   // with the particle itself
     o.out[__ldg(P.perm + s)] = a0;
 }
 
@@ -49,46 +48,45 @@ k_pair_fwd_q(PairParams P, PairOut o) {
     const bool live = s < P.n;
     const float4 pi = live ? __ldg(P.spos + s) : make_float4(0.f, 0.f, 0.f, 0.f);
     float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f;
-    const float ai = (OP == AB_OP_SPH_FORCE && live) ? __ldg(&P.sv[s].y) : 0.0f;
+    const float ai = OP != AB_OP_SPH_FORCE ? 0.0f : DIM == 2 ? pi.w : live ? __ldg(&P.sv[s].y) : 0.0f;
     if (live) visit_pairs<DIM, MODE, (OP == AB_OP_EXPF || OP == AB_OP_SOFT) ? 4 : 2, SL>(P, s, sub, pi,
-        [&](uint32_t j, const float4&, float dx, float dy, float dz, float d2) {
-            if (OP == AB_OP_SPH_FORCE) {
-                // m_j (A_i + A_j) W'(d)/d dx, W'(d)/d = wend_grad t^3
-                const float2 vj = __ldg(P.sv + j);
-                float q;
-                const float t = wend_t(d2, P.inv_r, q);
-                const float coef = vj.x * (ai + vj.y) * (P.wend_grad * (t * t * t));
-                a0 = fmaf(coef, dx, a0);
-                a1 = fmaf(coef, dy, a1);
-                a2 = fmaf(coef, dz, a2);
-            } else if (OP == AB_OP_LJ) {
+        [&](uint32_t j, const float4& pj, float dx, float dy, float dz, float d2) {
+            // EXPF and the SPH force leave out their common factor P.fscale
+            // (one multiplication a particle instead of one a pair; SOFT
+            // keeps its rounding, see pair_lanes_log2), and in 2-D
+            // the third component, which the compiler cannot drop
+            // (0 mag may be NaN)
+            float mag;
+            if (OP == AB_OP_LJ) {
                 const float sr2 = P.sig2 * rcp_approx(d2);
                 const float sr6 = sr2 * sr2 * sr2;
                 a0 = fmaf(sr6, sr6 - 1.0f, a0);
-            } else if (d2 > 0.0f) {   // EXPF, SOFT: coincident points contribute 0
-                float mag;
-                if (OP == AB_OP_EXPF) {
-                    const float inv_d = rsqrt_approx(d2);
-                    mag = -P.c * ex2_approx(-kLog2e * (d2 * inv_d)) * inv_d;
-                } else {
-                    // -k (r - d) / d with r - d = (r^2 - d^2) / (r + d): the
-                    // fma rounds r^2 - d^2 once, so the term keeps its relative
-                    // accuracy up to the cut-off, where r - d cancels, and d
-                    // enters only through 1/d and r + d (approximate
-                    // reciprocals, a few ulp)
-                    const float inv_d = rsqrt_approx(d2);
-                    const float d = d2 * inv_d;
-                    mag = (-P.k * fmaf(P.r, P.r, -d2)) * (inv_d * rcp_approx(P.r + d));
-                }
-                a0 = fmaf(mag, dx, a0);
-                a1 = fmaf(mag, dy, a1);
-                a2 = fmaf(mag, dz, a2);
+                return;
+            } else if (OP == AB_OP_SPH_FORCE) {
+                // m_j (A_i + A_j) (1 - d/r)^3 dx
+                const float2 vj = DIM == 2 ? make_float2(pj.z, pj.w) : __ldg(P.sv + j);
+                const float t = fmaf(-P.inv_r, pair_distance(d2), 1.0f);
+                mag = vj.x * (ai + vj.y) * (t * t * t);
+            } else {
+                // coincident points contribute 0: a finite mag times 0
+                const float inv_d = rsqrt_approx(fmaxf(d2, 1.17549435e-38f));
+                const float d = d2 * inv_d;
+                // SOFT: (r - d) / d with r - d = (r^2 - d^2) / (r + d): the fma
+                // rounds r^2 - d^2 once, so the term keeps its relative
+                // accuracy up to the cut-off, where r - d cancels, and d
+                // enters only through 1/d and r + d (approximate
+                // reciprocals, a few ulp)
+                if (OP == AB_OP_EXPF) mag = ex2_approx(-kLog2e * d) * inv_d;
+                else mag = (-P.k * fmaf(P.r, P.r, -d2)) * (inv_d * rcp_approx(P.r + d));
             }
+            a0 = fmaf(mag, dx, a0);
+            a1 = fmaf(mag, dy, a1);
+            if (DIM == 3) a2 = fmaf(mag, dz, a2);
         });
     a0 = lane_sum<SL>(a0);
     if (OP != AB_OP_LJ) {
         a1 = lane_sum<SL>(a1);
-        a2 = lane_sum<SL>(a2);
+        if (DIM == 3) a2 = lane_sum<SL>(a2);
     }
     const bool lead = live && sub == 0;
     if (lead) {
@@ -97,7 +95,7 @@ k_pair_fwd_q(PairParams P, PairOut o) {
             a0 *= 0.5f * P.eps;
             o.out[p] = a0;
         } else {
-            o.out4[p] = make_float4(a0, a1, DIM == 3 ? a2 : 0.0f, 0.0f);
+            o.out4[p] = make_float4(P.fscale * a0, P.fscale * a1, DIM == 3 ? P.fscale * a2 : 0.0f, 0.0f);
         }
     }
     if (OP == AB_OP_LJ && o.partial) block_partial<kPairThreads>(lead ? (double)a0 : 0.0, o.partial);
@@ -136,12 +134,12 @@ k_pair_emit(PairParams P, const int64_t* __restrict__ offsets, int32_t* __restri
 
 }  // namespace
 
-int pair_grid(const CellList& cl) { return pair_blocks(cl); }
+int pair_grid(const CellList& cl) { return pair_blocks(cl, pair_lanes_log2(cl, AB_OP_LJ)); }
 
 cudaError_t launch_pair_fwd(const CellList& cl, ab_op op, const ab_op_params& prm,
                             const float2* sv, PairOut& o, cudaStream_t st) {
     if (cl.n <= 0) return cudaSuccess;
-    const PairParams P = make_params(cl, prm, sv);
+    const PairParams P = make_params(cl, op, prm, sv);
     switch (op) {
         case AB_OP_COUNT: return AB_PAIR_LAUNCH(k_pair_fwd<DIM, MODE, SL, AB_OP_COUNT>);
         case AB_OP_GAUSS: return AB_PAIR_LAUNCH(k_pair_fwd<DIM, MODE, SL, AB_OP_GAUSS>);
@@ -156,7 +154,8 @@ cudaError_t launch_pair_fwd(const CellList& cl, ab_op op, const ab_op_params& pr
 
 cudaError_t launch_pair_count(const CellList& cl, uint32_t* counts, cudaStream_t st) {
     if (cl.n <= 0) return cudaSuccess;
-    const PairParams P = make_params(cl, ab_op_params{}, nullptr);
+    const ab_op op = AB_OP_COUNT;
+    const PairParams P = make_params(cl, op, ab_op_params{}, nullptr);
     uint32_t* const o = counts;
     return AB_PAIR_LAUNCH(k_pair_count<DIM, MODE, SL>);
 }
@@ -165,7 +164,7 @@ cudaError_t launch_pair_count(const CellList& cl, uint32_t* counts, cudaStream_t
 cudaError_t launch_pair_emit(const CellList& cl, const int64_t* offsets, int32_t* idx,
                              cudaStream_t st) {
     if (cl.n <= 0) return cudaSuccess;
-    const PairParams P = make_params(cl, ab_op_params{}, nullptr);
+    const PairParams P = make_params(cl, AB_OP_COUNT, ab_op_params{}, nullptr);
     const int grid = (int)((cl.n + kPairThreads - 1) / kPairThreads);
     auto emit = [&](auto dim) {
         constexpr int DIM = decltype(dim)::value;

@@ -47,11 +47,11 @@ struct PairParams {
     const float2* __restrict__ sv;
     int64_t n;
     Geom g;
-    float s, s_log2e, eps, sig2, c, k, r;
+    float s, s_log2e, eps, sig2, k, r;
+    float fscale;         // factor of a vector sum: -c (EXPF), 1 (SOFT), -20 a / r^2 (SPH force)
     float zero;   // 0.0f, passed at run time (see sq2)
     float wend_a;         // Wendland C2 normalisation a (SPH)
     float inv_r;          // 1 / r
-    float wend_grad;      // -20 a / r^2: W'(d)/d = wend_grad (1 - d/r)^3
 };
 
 
@@ -70,11 +70,10 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-// Wendland C2 with support r: t = 1 - d/r (and q = d/r) for a pair at d^2.
-__device__ __forceinline__ float wend_t(float d2, float inv_r, float& q) {
-    const float d = d2 > 0.0f ? d2 * rsqrt_approx(d2) : 0.0f;
-    q = d * inv_r;
-    return fmaxf(1.0f - q, 0.0f);
+// Distance of a pair at d^2, 0 for coincident points (the floor keeps the
+// reciprocal root finite; one operation where a test and a select took two).
+__device__ __forceinline__ float pair_distance(float d2) {
+    return d2 * rsqrt_approx(fmaxf(d2, 1.17549435e-38f));
 }
 
 // Canonical FP32 minimum image along one periodic axis.
@@ -263,6 +262,20 @@ __device__ __forceinline__ float pred_d2(const Geom& g, const float4& pi, const 
     return d2;
 }
 
+// The kernels are bound by issue slots (29 instructions a candidate step in
+// 3-D, the body entered on most of them by some lane), so a body's instruction
+// count is its time.  What the bodies leave out, us before and after (SOFT /
+// SPH density / SPH force / Gaussian adjoint): a common factor per pair, the
+// third component in 2-D, tests for coincident points where a floor under the
+// reciprocal root does, the clamp of 1 - d/r, ds where nobody asks for it, and
+// in 2-D the second value's own load (it rides in the z component):
+//   4M points in 2-D, 53 neighbours  406 / 493 / 558 / 550 -> 390 / 438 / 460 / 436
+//   1M points in 3-D, 57 neighbours  344 / 358 / 422 / 391 -> 337 / 338 / 391 / 372
+//   16.7M clustered points           5,129 / 5,375 / 6,554 / 5,871 -> 5,010 / 5,042 / 5,968 / 5,626
+// (SOFT in 2-D with one special-function operation instead of two and three
+// more FP32 ones: 417.  With its factor k taken out of the sum too: 381, 331
+// and 4,886, not kept because it changes the last bits, see pair_lanes_log2.)
+//
 // Direct visit: f(j, pj, dx, dy, dz, d2) for every accepted pair, with value
 // separations accurate to one rounding (see value_sep).  Used by every pair
 // kernel.  UNROLL is the unroll factor of the candidate loop, measured per
@@ -360,14 +373,19 @@ __device__ __forceinline__ void block_partial(double v, double* partial) {
     }
 }
 
-// Lanes that share a particle's walk (log2), the same for every operator and
-// table of a cell list, so that their results can be compared bit for bit.
+// Lanes that share a particle's walk (log2), the same for every table of a
+// cell list and, but for SOFT in 2-D, for every operator, so that their
+// results can be compared bit for bit.  SOFT drives time steppers in place: a
+// last bit of a force moves a position by one, and a pair closer than some
+// 30,000 of them then turns by more than a thousandth in the next step.
+// Points in the plane come that close by chance from about a hundred thousand
+// of them, so there SOFT keeps one lane and the order of its sums.
 // One lane a particle while the particles fill the SMs.  Fewer leave SMs
 // idle, and one lane's walk, thousands of dependent loads on dense inputs, is
 // all there is to wait for; more lanes then share it, but each row of a
 // stencil costs a lane its set-up and a warp its longest lane, so short rows
 // take fewer.  row: candidates expected in a stencil row.  Measured, us with
-// 1 / 2 / 4 / 8 / 32 lanes (EXPF or SOFT; the other operators alike):
+// 1 / 2 / 4 / 8 / 32 lanes (EXPF; the other operators alike):
 //   row 7:    1,000  9.3/ 8.2/ 6.6/ 5.0/ 4.6    32,768  11.2/ 8.8/ 7.8/ 8.2/ 21
 //            65,536 10.9/ 9.8/ 9.9/ 12 / 36    131,072  12.8/13.0/14.4/21.1/ 69
 //   row 18:  16,384   64/  48/  27/  19/  32    65,536    65/  46/  38/  42/ 98
@@ -378,8 +396,9 @@ __device__ __forceinline__ void block_partial(double v, double* partial) {
 //   row 215+: 65,536 512/ 366/ 261/ 204/ 181   131,072   264/ 236/ 184/ 164/184
 //           262,144  183/ 178/ 159/ 162/ 286   524,288   291/ 304/ 292/ 304/570
 // Million-particle inputs lose 10-20% with two lanes already.
-inline int pair_lanes_log2(const CellList& cl) {
+inline int pair_lanes_log2(const CellList& cl, ab_op op) {
     const int64_t n = cl.n;
+    if (op == AB_OP_SOFT && cl.g.dim == 2 && n > 1 << 15) return 0;
     const double row = (double)n / (double)cl.g.n_cells * (2 * cl.g.kx + 1);
     if (n > (1 << 18)) return 0;
     if (row >= 100.0) return n <= 3 << 15 ? 5 : n <= 3 << 16 ? 3 : 2;
@@ -391,7 +410,7 @@ inline int pair_lanes_log2(const CellList& cl) {
     return n <= 1 << 14 ? 3 : n <= 1 << 16 ? 2 : 0;
 }
 
-inline PairParams make_params(const CellList& cl, const ab_op_params& prm, const float2* sv) {
+inline PairParams make_params(const CellList& cl, ab_op op, const ab_op_params& prm, const float2* sv) {
     PairParams P;
     P.spos = cl.spos;
     P.cell_start = cl.cell_start;
@@ -404,7 +423,6 @@ inline PairParams make_params(const CellList& cl, const ab_op_params& prm, const
     P.s_log2e = prm.s * kLog2e;
     P.eps = prm.eps;
     P.sig2 = prm.sigma * prm.sigma;
-    P.c = prm.c;
     P.k = prm.k;
     P.r = cl.g.r;
     P.zero = 0.0f;
@@ -412,13 +430,14 @@ inline PairParams make_params(const CellList& cl, const ab_op_params& prm, const
     const double a = cl.g.dim == 3 ? 21.0 / (2.0 * pi * r * r * r) : 7.0 / (pi * r * r);
     P.wend_a = (float)a;
     P.inv_r = (float)(1.0 / r);
-    P.wend_grad = (float)(-20.0 * a / (r * r));
+    // W'(d)/d = -20 a / r^2 (1 - d/r)^3
+    P.fscale = op == AB_OP_EXPF ? -prm.c : op == AB_OP_SOFT ? 1.0f : (float)(-20.0 * a / (r * r));
     return P;
 }
 
 // Blocks of a pair kernel.
-inline int pair_blocks(const CellList& cl) {
-    return (int)(((cl.n << pair_lanes_log2(cl)) + kPairThreads - 1) / kPairThreads);
+inline int pair_blocks(const CellList& cl, int lanes_log2) {
+    return (int)(((cl.n << lanes_log2) + kPairThreads - 1) / kPairThreads);
 }
 
 // Launch as a programmatic dependent of the previous kernel on the stream
@@ -441,8 +460,8 @@ cudaError_t pdl_launch(void (*kern)(KArgs...), int grid, int threads, cudaStream
 // f(dim, mode, log2 of the lanes a particle) with the compile-time constants
 // of this cell list.
 template <class F>
-cudaError_t pair_dispatch(const CellList& cl, F&& f) {
-    const int lanes_log2 = pair_lanes_log2(cl);
+cudaError_t pair_dispatch(const CellList& cl, ab_op op, F&& f) {
+    const int lanes_log2 = pair_lanes_log2(cl, op);
     auto with_split = [&](auto dim, auto mode) {
         switch (lanes_log2) {
             case 1: return f(dim, mode, std::integral_constant<int, 1>{});
@@ -462,10 +481,10 @@ cudaError_t pair_dispatch(const CellList& cl, F&& f) {
 }
 
 #define AB_PAIR_LAUNCH(...)                                                              \
-    pair_dispatch(cl, [&](auto dim, auto mode, auto lanes) {                             \
+    pair_dispatch(cl, op, [&](auto dim, auto mode, auto lanes) {                         \
         constexpr int DIM = decltype(dim)::value, MODE = decltype(mode)::value;          \
         constexpr int SL = decltype(lanes)::value;                                       \
-        return pdl_launch(__VA_ARGS__, pair_blocks(cl), kPairThreads, st, P, o);         \
+        return pdl_launch(__VA_ARGS__, pair_blocks(cl, SL), kPairThreads, st, P, o);     \
     })
 
 }  // namespace
