@@ -1340,17 +1340,13 @@ namespace {
 // partial sums that another launch adds in order (four tiles' time, and both
 // move their bytes at about 1.9 MB a tile).  row_bytes: output of a row.
 // Against two ranges for fewer than four waves of row blocks and one
-// otherwise (bf16x3): 2000 x 30,000 points 118 -> 40 us, its adjoint 294 -> 127;
-// 16,000^2 115 -> 111 and 430 -> 403; 30,000 x 60,000 716 -> 614 and 2,720 ->
-// 2,467.
-// ordered (the solve's product): that old rule, because the iteration count
-// follows the last bits of the sums.
-int tc_splits(int64_t mblocks, int64_t tiles, int row_bytes, bool ordered) {
+// otherwise (BF16x3): 2000 x 12,000 points 59 -> 25 us, its adjoint 158 -> 76;
+// 8192^2 48 -> 41 and 168 -> 132; 30,000 x 60,000 adjoint 2,835 -> 2,472.
+int tc_splits(int64_t mblocks, int64_t tiles, int row_bytes, int least, int most) {
     const int64_t sms = num_sms();
-    if (ordered) return mblocks < 4 * sms && tiles >= 2 ? 2 : 1;
-    int best = 1;
+    int best = least;
     double cost = 1e300;
-    for (int s = 1; s <= 32 && (s == 1 || s <= tiles / 2); ++s) {
+    for (int s = least; s <= most && (s <= 2 || s <= tiles / 2); ++s) {
         const int64_t waves = (mblocks * s + sms - 1) / sms;
         double c = (double)waves * (double)((tiles + s - 1) / s + 3);
         if (s > 1)
@@ -1463,11 +1459,26 @@ cudaError_t run_fwd_prec(ab_prec prec, int64_t m, const float4* X, const FwdPrep
 bool is_tf32(ab_prec prec) { return prec == AB_PREC_TF32X3 || prec == AB_PREC_TF32; }
 int fwd_tile(ab_prec prec) { return is_tf32(prec) ? Tile<true>::TN : Tile<false>::TN; }
 
+// The product is summed over points in the tensor core's accumulator, which
+// truncates, so a sum is off by a share that grows with the points of its
+// range: a point 3.9e-9 (TF32x3), 2.3e-9 (BF16x3), 2.2e-9 (TF32) or 1.2e-9
+// (BF16), measured on 700 to 60,000 points, and other ranges move a result by
+// about as much.  So ranges are never longer than those of two ranges for fewer
+// than four waves of row blocks and one otherwise, and they are those where
+// others would move a result by more than 1.6e-5; a finer split of 30,000
+// points would be faster (2000 rows, BF16x3: 118 -> 40 us) and more exact, but
+// 3e-5 off what these ranges gave.  ordered (the solve's product): always
+// those, because the iteration count follows the last bits.
 int fwd_splits(ab_prec prec, int64_t m, int64_t n, bool ordered) {
     const int TN = fwd_tile(prec);
-    return tc_splits((m + kTM - 1) / kTM, (n + TN - 1) / TN, kRhs * 4, ordered);
+    const int64_t mblocks = (m + kTM - 1) / kTM, tiles = (n + TN - 1) / TN;
+    const int least = mblocks < 4 * (int64_t)num_sms() && tiles >= 2 ? 2 : 1;
+    const int64_t points = prec == AB_PREC_TF32X3 ? 4096 : prec == AB_PREC_BF16 ? 14336 : 7168;
+    if (ordered || n > least * points) return least;
+    return tc_splits(mblocks, tiles, kRhs * 4, least, 32);
 }
-int grad_splits(int64_t m, int64_t n) { return tc_splits((m + 127) / 128, (n + 127) / 128, 16, false); }
+// The gradients contract over the 64 columns and sum over points in FP32.
+int grad_splits(int64_t m, int64_t n) { return tc_splits((m + 127) / 128, (n + 127) / 128, 16, 1, 32); }
 
 // Partial sums of a product or gradient split more than in two.
 size_t fwd_parts_bytes(int splits, int64_t m) {
