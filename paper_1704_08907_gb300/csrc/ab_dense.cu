@@ -29,11 +29,11 @@
 // Bound: the FP32 pipe (7 + R operations a pair for values, 12 + R for
 // gradients, 128 a clock per SM).  Measured against the tile form, forward /
 // whole adjoint, us (and the forward's time at the pipe's rate):
-//   65,536 x 65,536, 64 columns   16,129 / 67,786 -> 12,213 / 35,809  (8,038)
-//   65,536 x 65,536,  1 column    16,042 / 66,625 ->  1,018 /  3,516    (906)
-//   16,384 x 16,384, 32 columns    1,465 /  5,851 ->    445 /  1,263    (276)
-//    5,001 x 12,345, 16 columns    1,102 /  2,783 ->     80 /    211     (37)
-//    2,000 x 30,000,  1 column     2,649 /  4,479 ->     32 /     87     (13)
+//   65,536 x 65,536, 64 columns   16,129 / 67,786 -> 10,921 / 33,158  (8,038)
+//   65,536 x 65,536,  1 column    16,042 / 66,625 ->  1,018 /  3,514    (906)
+//   16,384 x 16,384, 32 columns    1,465 /  5,851 ->    371 /  1,147    (276)
+//    5,001 x 12,345, 16 columns    1,102 /  2,783 ->     62 /    183     (37)
+//    2,000 x 30,000,  1 column     2,649 /  4,479 ->     31 /     83     (13)
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -109,6 +109,16 @@ __global__ void __launch_bounds__(kOwnThreads, OCC)
 k_dense_own(OwnArgs a) {
     static_assert(I % 2 == 0 && (R & (R - 1)) == 0, "rows in pairs, columns a power of two");
     constexpr int CH = R > 32 ? 64 : 128;     // points a stage
+    // Points a turn of the loop, so that loads and exponentials of some run
+    // under the products of others.  32 columns leave no registers for a
+    // second point's products: values alone then evaluate the next point's K
+    // under this point's products (PIPE).  16,384^2 pairs, forward / adjoint,
+    // us, with 4, 2 (8 and 16 columns) and 1 (32) points a turn -> this:
+    //   4 columns 107 / 350 -> 98 / 345     8: 147 / 496 -> 138 / 469
+    //   16: 249 / 753 -> 225 / 704          32: 444 / 1,260 -> 405 / 1,226
+    // (PIPE at 16 columns 227-235, more or fewer resident blocks no better.)
+    constexpr int TURN = R >= 32 ? (GRAD ? 2 : 1) : R >= 2 ? 8 : 4;
+    constexpr bool PIPE = VAL && !GRAD && R >= 32;
     constexpr int NP = I / 2;                 // row pairs
     constexpr int R2 = R > 1 ? R / 2 : 1;     // column pairs
     __shared__ __align__(16) float4 Ys[2][CH];
@@ -123,6 +133,13 @@ k_dense_own(OwnArgs a) {
     const int64_t j_begin = a.n * blockIdx.y / gridDim.y;
     const int64_t j_end = a.n * (blockIdx.y + 1) / gridDim.y;
 
+    // Aligned rows of whole float4s are copied, read and written 16 bytes at a
+    // time: a warp's 4-byte accesses at a row's stride cost a sector each (16,384^2
+    // pairs, forward / adjoint, us: 8 columns 138 / 471 -> 137 / 461, 16: 225 /
+    // 705 -> 213 / 680, 32: 404 / 1,227 -> 371 / 1,147; 5,001 x 12,345 in 45
+    // ranges with 16: 73 / 198 -> 62 / 183.  4 columns lose, 99 -> 102.)
+    auto wide = [&](const float* q) { return a.nrhs % 4 == 0 && ((uintptr_t)q & 15u) == 0; };
+
     uint64_t ox[NP], oy[NP], oz[NP];   // owned points, rows (2p, 2p + 1) packed
     uint64_t av[GRAD ? I : 1][R2];     // GRAD: their weights (R = 1: in the low half)
 #pragma unroll
@@ -132,7 +149,16 @@ k_dense_own(OwnArgs a) {
         for (int u = 0; u < 2; ++u) {
             const int64_t row = row0 + (2 * p + u) * kOwnThreads;
             o[u] = row < a.m ? __ldg(a.O + row) : make_float4(0.f, 0.f, 0.f, 0.f);
-            if (GRAD) {
+            if (GRAD && R >= 8 && wide(a.A)) {
+#pragma unroll
+                for (int c = 0; c < R2; c += 2) {
+                    const float4 w = row < a.m && 2 * c < nc
+                                         ? __ldg(reinterpret_cast<const float4*>(a.A + row * a.nrhs + 2 * c))
+                                         : make_float4(0.f, 0.f, 0.f, 0.f);
+                    av[2 * p + u][c] = f2p(w.x, w.y);
+                    av[2 * p + u][c + 1 < R2 ? c + 1 : c] = f2p(w.z, w.w);
+                }
+            } else if (GRAD) {
 #pragma unroll
                 for (int c = 0; c < R2; ++c) {
                     const float* q = a.A + row * a.nrhs + 2 * c;
@@ -161,6 +187,17 @@ k_dense_own(OwnArgs a) {
             const bool live = j0 + q < j_end;
             cp_async16((uint32_t)__cvta_generic_to_shared(&Ys[b][q]), a.P + (live ? j0 + q : 0), live);
         }
+        if (R >= 8 && wide(a.B)) {
+#pragma unroll 4
+            for (int e = t; e < CH * R / 4; e += kOwnThreads) {
+                const int jj = e / (R / 4 ? R / 4 : 1), c = e % (R / 4 ? R / 4 : 1) * 4;
+                const bool live = j0 + jj < j_end && c < nc;
+                cp_async16((uint32_t)__cvta_generic_to_shared(&Bs[b][4 * e]),
+                           a.B + (live ? (j0 + jj) * a.nrhs + c0 + c : 0), live);
+            }
+            cp_async_commit();
+            return;
+        }
 #pragma unroll 4
         for (int k = 0; k < CH * R / kOwnThreads; ++k) {
             const int e = k * kOwnThreads + t;
@@ -182,7 +219,45 @@ k_dense_own(OwnArgs a) {
         const int cnt = (int)(j_end - j0 < CH ? j_end - j0 : CH);
         const float4* __restrict__ Yb = Ys[b];
         const float* __restrict__ Bb = Bs[b];
-#pragma unroll (R >= 32 ? 1 : R >= 8 ? 2 : 4)
+        if constexpr (PIPE) {
+            auto kernel = [&](int j, uint64_t (&k)[NP]) {
+                const float4 y = Yb[j];
+                const uint64_t yx = f2p(y.x, y.x), yy = f2p(y.y, y.y), yz = f2p(y.z, y.z);
+#pragma unroll
+                for (int p = 0; p < NP; ++p) {
+                    const uint64_t dx = fsub2(ox[p], yx), dy = fsub2(oy[p], yy), dz = fsub2(oz[p], yz);
+                    const uint64_t d2 = ffma2(dz, dz, ffma2(dy, dy, fmul2(dx, dx)));
+                    float e0, e1;
+                    f2u(fmul2(d2, ns2), e0, e1);
+                    k[p] = f2p(ex2f(e0), ex2f(e1));
+                }
+            };
+            uint64_t k2[NP];
+            kernel(0, k2);
+#pragma unroll 1
+            for (int j = 0; j < cnt; ++j) {
+                uint64_t next[NP];
+                kernel(j + 1 < CH ? j + 1 : 0, next);   // the last one's is not used
+#pragma unroll
+                for (int c = 0; c < R2; c += 2) {
+                    const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(Bb + j * R + 2 * c);
+#pragma unroll
+                    for (int p = 0; p < NP; ++p) {
+                        float k0, k1;
+                        f2u(k2[p], k0, k1);
+                        const uint64_t kk0 = f2p(k0, k0), kk1 = f2p(k1, k1);
+                        v[2 * p][c] = ffma2(kk0, w.x, v[2 * p][c]);
+                        v[2 * p + 1][c] = ffma2(kk1, w.x, v[2 * p + 1][c]);
+                        v[2 * p][c + 1] = ffma2(kk0, w.y, v[2 * p][c + 1]);
+                        v[2 * p + 1][c + 1] = ffma2(kk1, w.y, v[2 * p + 1][c + 1]);
+                    }
+                }
+#pragma unroll
+                for (int p = 0; p < NP; ++p) k2[p] = next[p];
+            }
+            continue;
+        }
+#pragma unroll TURN
         for (int j = 0; j < cnt; ++j) {
             const float4 y = Yb[j];
             const uint64_t yx = f2p(y.x, y.x), yy = f2p(y.y, y.y), yz = f2p(y.z, y.z);
@@ -267,6 +342,14 @@ k_dense_own(OwnArgs a) {
                 float* q = a.val + ((int64_t)blockIdx.y * a.m + row) * a.nrhs + c0;
                 if (R == 1) {
                     q[0] = w[u];
+                } else if (R >= 8 && wide(a.val)) {
+#pragma unroll
+                    for (int c = 0; c < R2; c += 2) {
+                        float4 f;
+                        f2u(v[R > 1 ? 2 * p + u : 0][c], f.x, f.y);
+                        f2u(v[R > 1 ? 2 * p + u : 0][c + 1 < R2 ? c + 1 : c], f.z, f.w);
+                        if (2 * c < nc) *reinterpret_cast<float4*>(q + 2 * c) = f;
+                    }
                 } else {
 #pragma unroll
                     for (int c = 0; c < R2; ++c) {
