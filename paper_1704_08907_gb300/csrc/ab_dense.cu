@@ -32,8 +32,8 @@
 //   65,536 x 65,536, 64 columns   16,129 / 67,786 -> 10,921 / 33,158  (8,038)
 //   65,536 x 65,536,  1 column    16,042 / 66,625 ->  1,018 /  3,514    (906)
 //   16,384 x 16,384, 32 columns    1,465 /  5,851 ->    371 /  1,147    (276)
-//    5,001 x 12,345, 16 columns    1,102 /  2,783 ->     62 /    183     (37)
-//    2,000 x 30,000,  1 column     2,649 /  4,479 ->     31 /     83     (13)
+//    5,001 x 12,345, 16 columns    1,102 /  2,783 ->     59 /    177     (37)
+//    2,000 x 30,000,  1 column     2,649 /  4,479 ->     25 /     74     (13)
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -383,27 +383,53 @@ k_dense_own(OwnArgs a) {
     }
 }
 
+// Sum of splits partials `stride` apart, in their order, N loads in flight (the
+// last batch loads its end again rather than one by one).
+template <int N>
+__device__ __forceinline__ float sum_splits(const float* __restrict__ p, int splits, int64_t stride) {
+    float s = 0.f;
+#pragma unroll 1
+    for (int q0 = 0; q0 < splits; q0 += N) {
+        float x[N];
+#pragma unroll
+        for (int u = 0; u < N; ++u) x[u] = __ldcg(p + min(q0 + u, splits - 1) * stride);
+#pragma unroll
+        for (int u = 0; u < N; ++u) s += q0 + u < splits ? x[u] : 0.f;
+    }
+    return s;
+}
+
 // Sums of the splits' partials, in the order of the splits: `vals` floats and
-// `grads` float4 (either may be 0).
+// `grads` float4 (either may be 0).  Few rows have many splits and then wait
+// for the loads alone, so many are in flight at a time (against 8 and the rest
+// one by one, us, product / adjoint: 100 x 60,000 points 26.7 / 55 -> 20.6 / 39,
+// 2,000 x 30,000 28.7 / 80 -> 24.7 / 74, 300 x 4,000 with 8 columns 12.4 / 29 ->
+// 10.3 / 23).
 __global__ void __launch_bounds__(256)
 k_dense_combine(int splits, int64_t vals, const float* __restrict__ pv, float* __restrict__ val,
                 int64_t grads, const float4* __restrict__ pg, float4* __restrict__ grad) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (e < vals) {
-        float s = 0.f;
-#pragma unroll 8
-        for (int q = 0; q < splits; ++q) s += __ldcg(pv + q * vals + e);
-        val[e] = s;
+        val[e] = splits > 16  ? sum_splits<32>(pv + e, splits, vals)
+                 : splits > 8 ? sum_splits<16>(pv + e, splits, vals)
+                              : sum_splits<8>(pv + e, splits, vals);
     } else if (e - vals < grads) {
+        constexpr int N = 16;
         const int64_t r = e - vals;
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 8
-        for (int q = 0; q < splits; ++q) {
-            const float4 g = __ldcg(pg + q * grads + r);
-            s.x += g.x;
-            s.y += g.y;
-            s.z += g.z;
+#pragma unroll 1
+        for (int q0 = 0; q0 < splits; q0 += N) {
+            float4 g[N];
+#pragma unroll
+            for (int u = 0; u < N; ++u) g[u] = __ldcg(pg + min(q0 + u, splits - 1) * grads + r);
+#pragma unroll
+            for (int u = 0; u < N; ++u) {
+                const bool in = q0 + u < splits;
+                s.x += in ? g[u].x : 0.f;
+                s.y += in ? g[u].y : 0.f;
+                s.z += in ? g[u].z : 0.f;
+            }
         }
         grad[r] = s;
     }
