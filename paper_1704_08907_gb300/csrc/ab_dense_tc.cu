@@ -1469,13 +1469,19 @@ int fwd_tile(ab_prec prec) { return is_tf32(prec) ? Tile<true>::TN : Tile<false>
 // points would be faster (2000 rows, BF16x3: 118 -> 40 us) and more exact, but
 // 3e-5 off what these ranges gave.  ordered (the solve's product): always
 // those, because the iteration count follows the last bits.
+// More than two ranges write partial sums of up to kMaxParts bytes: a context's
+// first call also pays for that memory, about 2.5 us a megabyte (20,791 rows x
+// 7,812 points, 26 MB: first call 194 -> 272 us, later ones 143 -> 126).
+constexpr int64_t kMaxParts = int64_t(8) << 20;
+
 int fwd_splits(ab_prec prec, int64_t m, int64_t n, bool ordered) {
     const int TN = fwd_tile(prec);
     const int64_t mblocks = (m + kTM - 1) / kTM, tiles = (n + TN - 1) / TN;
     const int least = mblocks < 4 * (int64_t)num_sms() && tiles >= 2 ? 2 : 1;
     const int64_t points = prec == AB_PREC_TF32X3 ? 4096 : prec == AB_PREC_BF16 ? 14336 : 7168;
     if (ordered || n > least * points) return least;
-    return tc_splits(mblocks, tiles, kRhs * 4, least, 32);
+    const int64_t most = kMaxParts / ((m > 0 ? m : 1) * kRhs * 4);
+    return tc_splits(mblocks, tiles, kRhs * 4, least, (int)(most > 32 ? 32 : most > least ? most : least));
 }
 // The gradients contract over the 64 columns and sum over points in FP32.
 int grad_splits(int64_t m, int64_t n) { return tc_splits((m + 127) / 128, (n + 127) / 128, 16, 1, 32); }
