@@ -54,8 +54,8 @@ OPS_PER_PAIR_LJ_EG = 12
 # DRAM traffic of one k_pair_lj_eg<3,false> launch on this workload, from an
 # ncu --set full capture (dram__bytes_read.sum + dram__bytes_write.sum), valid
 # only for the kernel source it was taken on (None until captured).
-TRAFFIC_EG_BYTES = 35.54e6   # 29.28 MB read + 6.26 MB written
-TRAFFIC_SOURCE_SHA = "3b686070cc13ccc9"
+TRAFFIC_EG_BYTES = 35.45e6   # 29.22 MB read + 6.23 MB written
+TRAFFIC_SOURCE_SHA = "86c1f0575ff170b2"
 
 
 def pair_source_sha():
@@ -610,9 +610,9 @@ def oracle_sample_c3(w, nq, seed=23):
 # DRAM traffic of one k_pair_bwd<3,false,GAUSS> launch on the clustered
 # workload (ncu dram__bytes_read.sum + dram__bytes_write.sum), valid for the
 # kernel source whose hash is given (None until captured on that source).
-TRAFFIC_C3_BWD_BYTES = 942.84e6    # 550.14 MB read + 392.70 MB written (adjoint kernel)
-TRAFFIC_C3_VG_BYTES = 1129.44e6    # 612.22 MB read + 517.22 MB written (value and gradient)
-TRAFFIC_C3_SOURCE_SHA = "3b686070cc13ccc9"
+TRAFFIC_C3_BWD_BYTES = 942.08e6    # 549.40 MB read + 392.68 MB written (adjoint kernel)
+TRAFFIC_C3_VG_BYTES = 1129.62e6    # 612.22 MB read + 517.40 MB written (value and gradient)
+TRAFFIC_C3_SOURCE_SHA = "86c1f0575ff170b2"
 
 
 def also_c3(reps=5, oracle_fraction=64):

@@ -150,8 +150,9 @@ ab_status ab_sync(ab_ctx* ctx);
  * empty), the library keeps offsets of the occupied cells only, with a
  * bitmap of occupied cells to find them (about 0.25 bytes a cell plus 4 a
  * particle instead of 4 bytes a cell); the order and every result are the
- * same bit for bit.  Up to 2^21 particles, and for every compact table, the
- * build runs as one cooperative launch whose phases are separated by grid
+ * same bit for bit.  Few particles (8,192, and tables that fit shared memory
+ * beside them) are built by one block.  Up to 2^21 particles, and for every
+ * compact table, the build runs as one cooperative launch whose phases are separated by grid
  * barriers with bounded waits (a wait that gives up is reported by ab_sync
  * as AB_ERR_TIMEOUT); larger dense builds run as a sequence of kernels.
  *   dom:  host pointer to the domain (copied).
@@ -329,8 +330,9 @@ ab_status ab_bd_step(ab_ctx* ctx, const ab_domain* dom, int64_t n,
  * linear system of RBF interpolation with a nugget and of the Gaussian-
  * process posterior mean (paper Sec. 1.1; Rasmussen and Williams, Ch. 2).
  * Conjugate gradients (Hestenes and Stiefel), one independent iteration per
- * right-hand side, from W = 0; each iteration is one ab_kernel_matvec of the
- * chosen precision plus per-column FP64 inner products reduced in a fixed
+ * right-hand side, from W = 0; each iteration is one product of the chosen
+ * precision, summed in a fixed order of its own (one chain in increasing
+ * index for FP32), plus per-column FP64 inner products reduced in a fixed
  * order (run-to-run deterministic).  A column stops when
  * ||r|| <= tol ||b|| (r the recurrence residual); the call returns when all
  * have stopped or after max_iter iterations.
@@ -342,7 +344,10 @@ ab_status ab_bd_step(ab_ctx* ctx, const ab_domain* dom, int64_t n,
  *   W:      device float32[n][nrhs], the solution (overwritten).
  *   iters, relres: optional host outputs, the iterations run and the largest
  *           ||r||/||b|| over the columns.
- * Synchronises the context's stream once per iteration (the stopping test).
+ * Synchronises the context's stream before it returns, and once per iteration
+ * (the stopping test) except for FP32 systems of up to 4 columns and 64 rows
+ * an SM, which run in one cooperative launch with bounded waits (one that
+ * gives up is reported by ab_sync as AB_ERR_TIMEOUT, W undefined).
  * Errors: AB_ERR_INVALID_ARG, AB_ERR_ALIAS (W overlaps X or B),
  * AB_ERR_UNSUPPORTED, AB_ERR_OOM, AB_ERR_CUDA. */
 ab_status ab_kernel_solve(ab_ctx* ctx, int64_t n, const float* X, int32_t nrhs,
