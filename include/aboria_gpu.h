@@ -151,7 +151,7 @@ ab_status ab_sync(ab_ctx* ctx);
  * bitmap of occupied cells to find them (about 0.25 bytes a cell plus 4 a
  * particle instead of 4 bytes a cell); the order and every result are the
  * same bit for bit.  Few particles (8,192, and tables that fit shared memory
- * beside them) are built by one block.  Up to 2^21 particles, and for every
+ * beside them) are built by one block, up to 16,384 by a cluster of 16.  Up to 2^21 particles, and for every
  * compact table, the build runs as one cooperative launch whose phases are separated by grid
  * barriers with bounded waits (a wait that gives up is reported by ab_sync
  * as AB_ERR_TIMEOUT); larger dense builds run as a sequence of kernels.

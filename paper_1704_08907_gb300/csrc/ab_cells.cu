@@ -337,6 +337,7 @@ k_reduce_partials(const double* __restrict__ partial, int count, double* __restr
 // sorted order is the dense table's bit for bit.
 // ---------------------------------------------------------------------------
 constexpr int kCoopThreads = 1024;
+constexpr int kClusterMax = 16;        // blocks of the build over a cluster
 constexpr int kCoopBarWords = 4;        // barrier words at the start of the scratch (zeroed once)
 constexpr int kCoopIlp = 4;             // particles per thread per loop trip
 constexpr int kCoopScanItems = 16;      // cells per thread per scan tile (4 x 16-byte loads)
@@ -879,6 +880,104 @@ k_build_small(CoopArgs a) {
     }
 }
 
+// The one-block build over a thread-block cluster, for the next sizes: a
+// particle a thread.  Each of the K blocks holds the counts, then the offsets,
+// of a K-th of the cells in shared memory, particles add and look up across the
+// cluster, and the unordered slots go through L2.  The same cell list as the
+// other forms, bit for bit.  Bound: four cluster barriers and as many round
+// trips (8,193 points 21.4 us by the cooperative form's five grid barriers ->
+// 11.4, 16,384 21.7 -> 13.7).
+template <class T>
+__device__ __forceinline__ uint32_t peer_addr(const T* p, uint32_t rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ uint32_t peer_add(uint32_t addr, uint32_t v) {
+    uint32_t r;
+    asm volatile("atom.relaxed.cluster.shared::cluster.add.u32 %0, [%1], %2;" : "=r"(r) : "r"(addr), "r"(v) : "memory");
+    return r;
+}
+__device__ __forceinline__ uint32_t peer_load(uint32_t addr) {
+    uint32_t r;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(r) : "r"(addr) : "memory");
+    return r;
+}
+__device__ __forceinline__ void peer_store(uint32_t addr, uint32_t v) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+template <int DIM, bool PACKED>
+__global__ void __launch_bounds__(kCoopThreads, 1)
+k_build_cluster(CoopArgs a) {
+    asm volatile("griddepcontrol.launch_dependents;");
+    extern __shared__ __align__(16) uint32_t s_dyn[];
+    __shared__ uint32_t s_warp[32], s_total[kClusterMax], s_base[kClusterMax];
+    const int n = (int)a.n, t = threadIdx.x;
+    const uint32_t nc1 = (uint32_t)a.nc1, K = gridDim.x, k = blockIdx.x;   // one cluster
+    const uint32_t share = (nc1 + K - 1) / K;
+    const uint32_t c_first = k * share < nc1 ? k * share : nc1;
+    const uint32_t mine = nc1 - c_first < share ? nc1 - c_first : share;
+    uint32_t* const slots = reinterpret_cast<uint32_t*>(a.tmp);
+    for (uint32_t c = t; c < mine; c += kCoopThreads) s_dyn[c] = 0u;
+    const int i = (int)k * kCoopThreads + t;      // the thread's particle
+    const float4 q = i < n ? load_pos<DIM, PACKED>(a.pos, i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    const uint32_t cell = particle_cell<DIM, PACKED>(a, q);
+    uint32_t rank = 0;
+    cluster_sync();     // every block's counts are zero
+    if (i < n) {
+        const uint32_t o = cell / share;
+        rank = peer_add(peer_addr(s_dyn + (cell - o * share), o), 1u);
+    }
+    cluster_sync();
+    {   // counts -> offsets within the block's cells: a run of entries per thread
+        const uint32_t per = (mine + kCoopThreads - 1) / kCoopThreads;
+        const uint32_t c0 = t * per, c1 = c0 + per < mine ? c0 + per : mine;
+        uint32_t sum = 0, total;
+        for (uint32_t c = c0; c < c1; ++c) sum += s_dyn[c];
+        uint32_t ex = block_excl_scan(sum, s_warp, &total);
+        for (uint32_t c = c0; c < c1; ++c) {
+            const uint32_t v = s_dyn[c];
+            s_dyn[c] = ex;
+            ex += v;
+        }
+        if (t < (int)K) peer_store(peer_addr(s_total + k, (uint32_t)t), total);
+    }
+    cluster_sync();
+    if (t < (int)K) {
+        uint32_t b = 0;
+        for (int o = 0; o < t; ++o) b += s_total[o];
+        s_base[t] = b;
+    }
+    __syncthreads();
+    for (uint32_t c = t; c < mine; c += kCoopThreads) a.cell_start[c_first + c] = s_dyn[c] + s_base[k];
+    auto offset = [&](uint32_t c) {
+        const uint32_t o = c / share;
+        return peer_load(peer_addr(s_dyn + (c - o * share), o)) + s_base[o];
+    };
+    const uint32_t lo = offset(cell), hi = offset(cell + 1u);
+    if (i < n) slots[lo + rank] = (uint32_t)i;
+    cluster_sync();     // the slots are written, and no block's shared memory is read any more
+    if (i >= n) return;
+    // stable rank: the members of the cell with a smaller original index
+    uint32_t r = 0, s = lo;
+    if (hi - lo >= 16) {            // crowded cells: four members a load
+        for (; s & 3u; ++s) r += ldcg_u32(slots + s) < (uint32_t)i ? 1u : 0u;
+#pragma unroll 4
+        for (; s + 4 <= hi; s += 4) {
+            const uint4 m = __ldcg(reinterpret_cast<const uint4*>(slots + s));
+            r += (m.x < (uint32_t)i) + (m.y < (uint32_t)i) + (m.z < (uint32_t)i) + (m.w < (uint32_t)i);
+        }
+    }
+#pragma unroll 4
+    for (; s < hi; ++s) r += ldcg_u32(slots + s) < (uint32_t)i ? 1u : 0u;
+    a.perm[lo + r] = (uint32_t)i;
+    a.spos[lo + r] = make_float4(q.x, q.y, DIM == 3 ? q.z : 0.0f, 0.0f);
+}
+
 // Dense offsets of a compact cell list (inspection and export).
 __global__ void __launch_bounds__(kThreads)
 k_expand_cells(int64_t nc1, const uint4* __restrict__ occ, const uint32_t* __restrict__ cstart,
@@ -982,7 +1081,8 @@ int auto_build_path(int64_t n, const Geom& g) {
 }
 
 // Particles and shared memory (offsets and slots) up to which the one-block
-// build is taken (8,192 points: 16 us against the cooperative form's 21).
+// build is taken where the cluster's is not (8,192 points: 16 us against the
+// cooperative form's 21).
 constexpr int64_t kSmallMaxN = 8192;
 constexpr size_t kSmallMaxSmem = 128 * 1024;
 
@@ -1007,6 +1107,43 @@ static cudaError_t launch_small(const CoopArgs& a, cudaStream_t st) {
                                      : go(k_build_small<DIM, PACKED, 8>);
 }
 
+// Particles, and shared memory for a block's cells, between which a cluster of
+// kClusterMax blocks builds (6,000 points 12.6 us by one block, 11.1 by the
+// cluster, 4,500 10.7 and 11.0; 24,000 with two a thread 20.1, 21.7 by the
+// cooperative form), unless cells hold more than 32 points on average, whose
+// slots few SMs would read through L2 (16,384 points, 28 a cell: 20.7 us, 23.6
+// by the cooperative form, 29.8 without the loads of four).
+constexpr int64_t kClusterMinN = 6144;
+constexpr int64_t kClusterMaxN = kClusterMax * kCoopThreads;   // a particle a thread
+constexpr size_t kClusterMaxSmem = 160 * 1024;
+
+static size_t cluster_smem(int64_t nc1) {
+    return (size_t)((nc1 + kClusterMax - 1) / kClusterMax) * sizeof(uint32_t);
+}
+
+template <int DIM, bool PACKED>
+static cudaError_t launch_cluster(const CoopArgs& a, cudaStream_t st) {
+    const size_t smem = cluster_smem(a.nc1);
+    void (*const kern)(CoopArgs) = k_build_cluster<DIM, PACKED>;
+    // attributes belong to the device: set on every launch
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess && smem > 40 * 1024)
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterMaxSmem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kClusterMax);
+    cfg.blockDim = dim3(kCoopThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = kClusterMax;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
 cudaError_t launch_build(CellList& cl, const float* pos, bool packed, Scratch& sc,
                          uint32_t* err, cudaStream_t st, const BuildOptions& opt) {
     const int64_t n = cl.n;
@@ -1023,6 +1160,22 @@ cudaError_t launch_build(CellList& cl, const float* pos, bool packed, Scratch& s
     const int path = opt.path == kPathAuto ? auto_build_path(n, cl.g) : opt.path;
     if (path == kPathRadix && radix_supported(n, nc))
         return launch_build_radix(cl, pos, packed, sc, err, st, opt);
+    if (!compact && opt.path == kPathAuto && opt.skip_block < 0 && n > kClusterMinN && n <= kClusterMaxN &&
+        n <= 32 * nc && cluster_smem(nc + 1) <= kClusterMaxSmem) {
+        CoopArgs a = {};
+        a.pos = pos;
+        a.n = n;
+        a.g = cl.g;
+        a.nc1 = nc + 1;
+        a.cell_start = cl.cell_start;
+        a.tmp = reinterpret_cast<uint2*>(cl.tmp);
+        a.perm = cl.perm;
+        a.spos = cl.spos;
+        const cudaError_t e = cl.g.dim == 3 ? (packed ? launch_cluster<3, true>(a, st) : launch_cluster<3, false>(a, st))
+                                            : (packed ? launch_cluster<2, true>(a, st) : launch_cluster<2, false>(a, st));
+        if (e == cudaSuccess) return e;
+        cudaGetLastError();   // no room for the cluster on this device: the forms below
+    }
     if (!compact && opt.path == kPathAuto && opt.skip_block < 0 && n <= kSmallMaxN &&
         small_smem(n, nc + 1) <= kSmallMaxSmem) {
         CoopArgs a = {};
