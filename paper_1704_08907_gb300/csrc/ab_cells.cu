@@ -280,6 +280,10 @@ constexpr int kRedThreads = 256;
 constexpr int kRedBlocks = 8;
 __global__ void __launch_bounds__(kRedThreads)
 k_reduce_partials(const double* __restrict__ partial, int count, double* __restrict__ out) {
+    // a block's shared memory may be written by the others only once it is
+    // known to run: arrive here, wait before the store, so that the barrier's
+    // latency lies under the loads
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     // launched as a programmatic dependent of the kernel that writes the
     // partials: wait until that grid has finished and its writes are visible
     // (returns at once without a prerequisite grid)
@@ -305,6 +309,7 @@ k_reduce_partials(const double* __restrict__ partial, int count, double* __restr
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = v;
     __syncthreads();
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
     if (threadIdx.x == 0) {
         double b = 0.0;
 #pragma unroll
