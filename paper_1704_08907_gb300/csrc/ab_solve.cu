@@ -59,7 +59,8 @@ __device__ __forceinline__ void col_partial(double v, int c, int nrhs, double* p
 
 // The step kernels are programmatic dependent launches of the kernel before
 // them: scheduled while it finishes, they wait here for its writes, and read
-// what it wrote from L2.
+// what it wrote from L2 (col too, which k_solve_finish writes while the next
+// one may already be resident).
 __device__ __forceinline__ void solve_dependent() {
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -109,7 +110,7 @@ k_solve_pap(int64_t n, int nrhs, const float* __restrict__ P, const float* __res
 // W += alpha p, R -= alpha (q + sigma^2 p); partial of the new r.r
 __global__ void __launch_bounds__(kCols * kRowLanes)
 k_solve_update(int64_t n, int nrhs, const float* __restrict__ P, const float* __restrict__ Q,
-               float sigma2, const Col* __restrict__ col, float* __restrict__ R,
+               float sigma2, const Col* col, float* __restrict__ R,
                float* __restrict__ W, double* __restrict__ partial) {
     solve_dependent();
     const int c = blockIdx.y * kCols + threadIdx.x;
@@ -117,8 +118,8 @@ k_solve_update(int64_t n, int nrhs, const float* __restrict__ P, const float* __
     row_range(n, r0, r1);
     double acc = 0.0;
     if (c < nrhs) {
-        const Col k = col[c];
-        const float alpha = (k.active && k.pap > 0.0) ? (float)(k.rs / k.pap) : 0.0f;
+        const double rs = __ldcg(&col[c].rs), pap = __ldcg(&col[c].pap);
+        const float alpha = (__ldcg(&col[c].active) && pap > 0.0) ? (float)(rs / pap) : 0.0f;
         for (int64_t i = r0 + threadIdx.y; i < r1; i += kRowLanes) {
             const int64_t e = i * nrhs + c;
             const float p = __ldcg(P + e);
@@ -134,18 +135,18 @@ k_solve_update(int64_t n, int nrhs, const float* __restrict__ P, const float* __
 
 // P = R + beta P (frozen columns: P = 0)
 __global__ void __launch_bounds__(kCols * kRowLanes)
-k_solve_dir(int64_t n, int nrhs, const float* __restrict__ R, const Col* __restrict__ col,
+k_solve_dir(int64_t n, int nrhs, const float* __restrict__ R, const Col* col,
             float* __restrict__ P) {
     solve_dependent();
     const int c = blockIdx.y * kCols + threadIdx.x;
     int64_t r0, r1;
     row_range(n, r0, r1);
     if (c >= nrhs) return;
-    const Col k = col[c];
-    const float beta = (float)k.beta;
+    const int active = __ldcg(&col[c].active);
+    const float beta = (float)__ldcg(&col[c].beta);
     for (int64_t i = r0 + threadIdx.y; i < r1; i += kRowLanes) {
         const int64_t e = i * nrhs + c;
-        P[e] = k.active ? fmaf(beta, __ldcg(P + e), __ldcg(R + e)) : 0.0f;
+        P[e] = active ? fmaf(beta, __ldcg(P + e), __ldcg(R + e)) : 0.0f;
     }
 }
 
@@ -155,7 +156,7 @@ k_solve_dir(int64_t n, int nrhs, const float* __restrict__ R, const Col* __restr
 // more, and all columns on one SM took longer than the rest of a step.
 __global__ void __launch_bounds__(32)
 k_solve_finish(const double* __restrict__ partial, int blocks, int nrhs, int what, double tol2,
-               Col* __restrict__ col, int* __restrict__ n_active) {
+               Col* col, int* __restrict__ n_active) {
     solve_dependent();
     const int c = blockIdx.x, lane = threadIdx.x;
     double t = 0.0;
@@ -163,7 +164,14 @@ k_solve_finish(const double* __restrict__ partial, int blocks, int nrhs, int wha
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
     if (lane != 0) return;
-    Col k = col[c];
+    Col k;
+    k.bb = __ldcg(&col[c].bb);
+    k.rs = __ldcg(&col[c].rs);
+    k.pap = __ldcg(&col[c].pap);
+    k.rs_new = __ldcg(&col[c].rs_new);
+    k.beta = __ldcg(&col[c].beta);
+    k.active = __ldcg(&col[c].active);
+    k.pad = 0;
     if (what == 0) {
         k.bb = t;
         k.rs = t;
