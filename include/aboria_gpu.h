@@ -36,7 +36,9 @@
  *  - The context owns its workspace (cell table, sorted copies, scan state)
  *    and grows it on demand with cudaMallocAsync on the context's stream
  *    (the device's default memory pool); AB_ERR_OOM leaves the context
- *    usable with its previous workspace.
+ *    usable with its previous workspace.  The dense calls (ab_kernel_matvec
+ *    and its adjoint) share no workspace between streams, and captured in a
+ *    graph they use an allocation of the graph's own.
  *  - Each call makes the context's device current while it runs and
  *    restores the caller's current device before it returns; a failure to
  *    select the device returns AB_ERR_CUDA.

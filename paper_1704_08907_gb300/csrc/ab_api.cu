@@ -65,6 +65,8 @@ struct ab_ctx {
     ab::BuildOptions build_opt;
     int coop_launch = 0;      // the device supports cooperative launches
     int table_mode = 0;       // testing: 0 automatic, 1 dense, 2 compact where allowed
+    unsigned long long dense_stream = 0;   // id of the stream that sc.dense_ws belongs to
+    cudaMemPool_t pool = nullptr;          // dense workspace of other streams (call_pool)
     uint32_t* d_err = nullptr;
     std::string last_error;
 };
@@ -216,21 +218,87 @@ ab_status ensure_scan(ab_ctx* c, int64_t items) {
     return AB_OK;
 }
 
-// Workspace of the FP32 dense walks' partial sums, or NULL, on which they run
-// unsplit (slower on few rows, never refused): when the memory is not to be
-// had, and under stream capture, where a captured call would keep a pointer
-// that a later, larger call frees.
-void* dense_scratch(ab_ctx* c, size_t need) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (need == 0) return nullptr;
-    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
+// Memory that the pool of call_pool keeps between calls; what it holds beyond
+// that goes back to the device at the next synchronisation.
+constexpr uint64_t kPoolKeepBytes = uint64_t(256) << 20;
+
+// The context's pool for the memory of single calls, made when first wanted
+// (NULL: the device's default pool).  Streams do not wait for one another to
+// reuse its memory.
+cudaMemPool_t call_pool(ab_ctx* c) {
+    if (c->pool) return c->pool;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = c->device;
+    if (cudaMemPoolCreate(&c->pool, &props) != cudaSuccess) {
         cudaGetLastError();
-        return nullptr;
+        return c->pool = nullptr;
     }
-    if (cap != cudaStreamCaptureStatusNone) return nullptr;
-    return grow(&c->sc.dense_ws, &c->sc.cap_dense_ws, need, c->stream) == cudaSuccess ? c->sc.dense_ws
-                                                                                     : nullptr;
+    uint64_t keep = kPoolKeepBytes;
+    int wait = 0;
+    if (cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
+        cudaMemPoolSetAttribute(c->pool, cudaMemPoolReuseAllowInternalDependencies, &wait) != cudaSuccess)
+        cudaGetLastError();
+    return c->pool;
 }
+
+// Workspace of one dense call.  A context's products may run on several
+// streams at once and inside graphs, and never share it:
+//  - The stream of the context's first dense call has a buffer that stays
+//    (streams are told apart by their ids: a handle may come back for a new
+//    stream while the old one's work still runs).
+//  - Other streams take the call's memory from a pool and give it back in
+//    stream order.  (Not for every call: making the pool takes 170 us of a
+//    context's first product, 2,000 x 30,000 points 66 -> 233 us.)
+//  - A captured call gets an allocation of the graph's own: a pointer of the
+//    context's would dangle once a later, larger call has replaced the buffer.
+class CallMemory {
+  public:
+    explicit CallMemory(ab_ctx* c) : c_(c) {}
+    ~CallMemory() {
+        if (own_) cudaFreeAsync(p_, c_->stream);
+    }
+    CallMemory(const CallMemory&) = delete;
+    CallMemory& operator=(const CallMemory&) = delete;
+    cudaError_t take(size_t bytes) {
+        if (bytes == 0) return cudaSuccess;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(c_->stream, &cap) != cudaSuccess) cudaGetLastError();
+        cudaMemPool_t pool = nullptr;
+        if (cap == cudaStreamCaptureStatusNone) {
+            unsigned long long id = 0;
+            const bool known = cudaStreamGetId(c_->stream, &id) == cudaSuccess;
+            if (!known) cudaGetLastError();
+            if (known && (!c_->sc.dense_ws || id == c_->dense_stream)) {
+                const cudaError_t e = grow(&c_->sc.dense_ws, &c_->sc.cap_dense_ws, bytes, c_->stream);
+                if (e == cudaSuccess) {
+                    c_->dense_stream = id;
+                    p_ = c_->sc.dense_ws;
+                }
+                return e;
+            }
+            pool = call_pool(c_);
+        }
+        const cudaError_t e = pool ? cudaMallocFromPoolAsync(&p_, bytes, pool, c_->stream)
+                                   : cudaMallocAsync(&p_, bytes, c_->stream);
+        own_ = e == cudaSuccess;
+        if (!own_) {
+            cudaGetLastError();
+            p_ = nullptr;
+        }
+        return e;
+    }
+    uint8_t* get() const { return (uint8_t*)p_; }
+
+  private:
+    ab_ctx* c_;
+    void* p_ = nullptr;
+    bool own_ = false;
+};
+
+size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 ab_status require_cells(ab_ctx* c) {
     if (!c->cl.valid)
@@ -306,6 +374,7 @@ ab_status ab_destroy(ab_ctx* c) {
     for (void* b : bufs)
         if (b) cudaFreeAsync(b, c->stream);
     cudaStreamSynchronize(c->stream);
+    if (c->pool) cudaMemPoolDestroy(c->pool);
     cudaFree(c->d_err);
     cudaGetLastError();
     delete c;
@@ -704,18 +773,19 @@ ab_status ab_kernel_matvec(ab_ctx* c, int64_t m, int64_t n, const float* X, cons
     ab::DeviceGuard dg(c->device);
     if (!dg.ok) return fail(c, AB_ERR_CUDA, "cannot make device %d current", c->device);
     cudaError_t e;
+    CallMemory mem(c);
     if (prec == AB_PREC_FP32) {
-        void* ws = dense_scratch(c, ab::dense_fwd_workspace_bytes(m, n, nrhs));
-        e = ab::launch_dense_fwd(m, n, (const float4*)X, (const float4*)Y, nrhs, W, s, out, ws,
+        // without the memory, unsplit (slower on few rows, never refused)
+        (void)mem.take(ab::dense_fwd_workspace_bytes(m, n, nrhs));
+        e = ab::launch_dense_fwd(m, n, (const float4*)X, (const float4*)Y, nrhs, W, s, out, mem.get(),
                                  c->stream);
     } else {
         if (nrhs != 64)
             return fail(c, AB_ERR_UNSUPPORTED, "tensor-core paths need nrhs == 64");
-        e = grow(&c->sc.dense_ws, &c->sc.cap_dense_ws, ab::dense_tc_workspace_bytes(m, n, prec, false),
-                 c->stream);
+        e = mem.take(ab::dense_tc_workspace_bytes(m, n, prec, false));
         if (e != cudaSuccess) return cuda_fail(c, e, "ab_kernel_matvec workspace");
         e = ab::launch_dense_tc_fwd(m, n, (const float4*)X, (const float4*)Y, nrhs, W, s, prec, out, false,
-                                    c->sc.dense_ws, c->d_err, c->stream);
+                                    mem.get(), c->d_err, c->stream);
     }
     if (e == cudaErrorNotSupported)
         return fail(c, AB_ERR_UNSUPPORTED, "precision not available for this shape");
@@ -760,15 +830,14 @@ ab_status ab_kernel_solve(ab_ctx* c, int64_t n, const float* X, int32_t nrhs, co
         }
     }
     e = grow(&c->sc.solve_ws, &c->sc.cap_solve_ws, ab::solve_workspace_bytes(n, nrhs), c->stream);
-    if (e == cudaSuccess && prec != AB_PREC_FP32)
-        e = grow(&c->sc.dense_ws, &c->sc.cap_dense_ws, ab::dense_tc_workspace_bytes(n, n, prec, true),
-                 c->stream);
+    CallMemory mem(c);
+    if (e == cudaSuccess && prec != AB_PREC_FP32) e = mem.take(ab::dense_tc_workspace_bytes(n, n, prec, true));
     if (e != cudaSuccess) return cuda_fail(c, e, "ab_kernel_solve workspace");
     const float4* X4 = (const float4*)X;
     const ab::SolveMatvec mv = [&](const float* P, float* Q) -> cudaError_t {
         if (prec == AB_PREC_FP32)
             return ab::launch_dense_fwd_ordered(n, n, X4, X4, nrhs, P, s, Q, c->stream);
-        return ab::launch_dense_tc_fwd(n, n, X4, X4, nrhs, P, s, prec, Q, true, c->sc.dense_ws, c->d_err,
+        return ab::launch_dense_tc_fwd(n, n, X4, X4, nrhs, P, s, prec, Q, true, mem.get(), c->d_err,
                                        c->stream);
     };
     e = ab::run_solve(n, nrhs, B, sigma2, tol, max_iter, W, c->sc.solve_ws, mv, &it, &rr, c->stream);
@@ -803,31 +872,32 @@ ab_status ab_kernel_matvec_bwd(ab_ctx* c, int64_t m, int64_t n, const float* X, 
     }
     ab::DeviceGuard dg(c->device);
     if (!dg.ok) return fail(c, AB_ERR_CUDA, "cannot make device %d current", c->device);
+    // the partials of ds first, then the kernels' workspace
+    CallMemory mem(c);
     double* partial = nullptr;
-    if (ds) {
-        const size_t count = prec == AB_PREC_FP32 ? ab::dense_partial_capacity(m, n, nrhs)
-                                                  : ab::dense_tc_partial_capacity(m, n);
-        if ((st = ensure_partial(c, count)) != AB_OK) return st;
-        partial = c->sc.partial;
-    }
     int pc = 0;
     cudaError_t e;
     if (prec == AB_PREC_FP32) {
-        void* ws = dense_scratch(c, ab::dense_bwd_workspace_bytes(
-                                        m, n, nrhs, dW != nullptr, dX != nullptr, dY != nullptr,
-                                        ds != nullptr));
+        const size_t pb = ds ? up256(ab::dense_partial_capacity(m, n, nrhs) * sizeof(double)) : 0;
+        const size_t wb = ab::dense_bwd_workspace_bytes(m, n, nrhs, dW != nullptr, dX != nullptr,
+                                                        dY != nullptr, ds != nullptr);
+        const bool split = wb > 0 && mem.take(pb + wb) == cudaSuccess;
+        if (!split && (e = mem.take(pb)) != cudaSuccess) return cuda_fail(c, e, "ab_kernel_matvec_bwd workspace");
+        if (ds) partial = (double*)mem.get();
         e = ab::launch_dense_bwd(m, n, (const float4*)X, (const float4*)Y, nrhs, W, s, G, dW,
-                                 (float4*)dX, (float4*)dY, partial, &pc, ws, c->stream);
+                                 (float4*)dX, (float4*)dY, partial, &pc, split ? mem.get() + pb : nullptr,
+                                 c->stream);
     } else {
         if (nrhs != 64)
             return fail(c, AB_ERR_UNSUPPORTED, "tensor-core paths need nrhs == 64");
-        e = grow(&c->sc.dense_ws, &c->sc.cap_dense_ws,
-                 ab::dense_tc_bwd_workspace_bytes(m, n, prec, dW != nullptr, dX != nullptr, dY != nullptr),
-                 c->stream);
-        if (e == cudaSuccess)
-            e = ab::launch_dense_tc_bwd(m, n, (const float4*)X, (const float4*)Y, W, s, prec, G, dW,
-                                        (float4*)dX, (float4*)dY, partial, &pc, c->sc.dense_ws, c->d_err,
-                                        c->stream);
+        const size_t pb = ds ? up256(ab::dense_tc_partial_capacity(m, n) * sizeof(double)) : 0;
+        e = mem.take(pb + ab::dense_tc_bwd_workspace_bytes(m, n, prec, dW != nullptr, dX != nullptr,
+                                                           dY != nullptr));
+        if (e != cudaSuccess) return cuda_fail(c, e, "ab_kernel_matvec_bwd workspace");
+        if (ds) partial = (double*)mem.get();
+        e = ab::launch_dense_tc_bwd(m, n, (const float4*)X, (const float4*)Y, W, s, prec, G, dW,
+                                    (float4*)dX, (float4*)dY, partial, &pc, mem.get() + pb, c->d_err,
+                                    c->stream);
     }
     if (e == cudaErrorNotSupported)
         return fail(c, AB_ERR_UNSUPPORTED, "precision not available for this shape");

@@ -80,7 +80,7 @@ struct Scratch {
     size_t cap_partial = 0;
     uint32_t* counts = nullptr;       // pair-list counts (user order)
     size_t cap_counts = 0;
-    uint8_t* dense_ws = nullptr;      // tensor-core operand images
+    uint8_t* dense_ws = nullptr;      // dense operands and partial sums (of one stream)
     size_t cap_dense_ws = 0;
     uint8_t* solve_ws = nullptr;      // CG vectors and scalars
     size_t cap_solve_ws = 0;
