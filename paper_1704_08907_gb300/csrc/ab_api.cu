@@ -586,7 +586,7 @@ ab_status ab_pair_sum(ab_ctx* c, ab_op op, const ab_op_params* prm, const float*
     o.out4 = vec ? (float4*)out : nullptr;
     const int grid = ab::pair_grid(c->cl);
     if (op == AB_OP_LJ && energy) {
-        if ((s = ensure_partial(c, (size_t)grid)) != AB_OK) return s;
+        if ((s = ensure_partial(c, ab::pair_partial_capacity(n))) != AB_OK) return s;
         o.partial = c->sc.partial;
         o.partial_count = grid;
     }
@@ -624,7 +624,7 @@ static ab_status energy_grad_impl(ab_ctx* c, ab_op op, const ab_op_params* prm, 
     else o.grad_pos = (float4*)grad;
     const int grid = ab::pair_grid(c->cl);
     if (energy) {
-        if ((s = ensure_partial(c, (size_t)grid)) != AB_OK) return s;
+        if ((s = ensure_partial(c, ab::pair_partial_capacity(n))) != AB_OK) return s;
         o.partial = c->sc.partial;
         o.partial_count = grid;
     }
@@ -691,7 +691,7 @@ static ab_status pair_bwd_impl(ab_ctx* c, ab_op op, const ab_op_params* prm, con
     const int grid = ab::pair_grid(c->cl);
     double* red = op == AB_OP_GAUSS ? grad_s : (value ? energy : nullptr);
     if (red) {
-        if ((s = ensure_partial(c, (size_t)grid)) != AB_OK) return s;
+        if ((s = ensure_partial(c, ab::pair_partial_capacity(n))) != AB_OK) return s;
         o.partial = c->sc.partial;
         o.partial_count = grid;
     }

@@ -159,6 +159,11 @@ struct PairOut {
     int partial_count = 0;
 };
 AB_HIDDEN int pair_grid(const CellList& cl);   // blocks of a pair kernel (block partials)
+// Block partials of any pair kernel on at most n particles.  It follows n alone,
+// not the lanes that this lattice's particles get, so that a context's buffer
+// is replaced only by calls with more particles: the particle buffers are
+// replaced then too, and a captured call may hold either.
+AB_HIDDEN size_t pair_partial_capacity(int64_t n);
 AB_HIDDEN int num_sms();   // SM count of the current device
 AB_HIDDEN cudaError_t launch_pair_fwd(const CellList& cl, ab_op op,
                                       const ab_op_params& prm, const float2* sv,

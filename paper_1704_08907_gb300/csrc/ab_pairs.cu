@@ -136,6 +136,12 @@ k_pair_emit(PairParams P, const int64_t* __restrict__ offsets, int32_t* __restri
 
 int pair_grid(const CellList& cl) { return pair_blocks(cl, pair_lanes_log2(cl, AB_OP_LJ)); }
 
+size_t pair_partial_capacity(int64_t n) {
+    const int64_t split = n < kMaxSplitN ? n : kMaxSplitN;
+    const int64_t threads = n > split << kMaxLanesLog2 ? n : split << kMaxLanesLog2;
+    return (size_t)((threads + kPairThreads - 1) / kPairThreads);
+}
+
 cudaError_t launch_pair_fwd(const CellList& cl, ab_op op, const ab_op_params& prm,
                             const float2* sv, PairOut& o, cudaStream_t st) {
     if (cl.n <= 0) return cudaSuccess;

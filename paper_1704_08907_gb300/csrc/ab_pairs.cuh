@@ -396,12 +396,16 @@ __device__ __forceinline__ void block_partial(double v, double* partial) {
 //   row 215+: 65,536 512/ 366/ 261/ 204/ 181   131,072   264/ 236/ 184/ 164/184
 //           262,144  183/ 178/ 159/ 162/ 286   524,288   291/ 304/ 292/ 304/570
 // Million-particle inputs lose 10-20% with two lanes already.
+// No rule gives more than kMaxSplitN << kMaxLanesLog2 lanes in all, or a
+// particle more than 2^kMaxLanesLog2 (pair_partial_capacity builds on it).
+constexpr int64_t kMaxSplitN = 3 << 15;
+constexpr int kMaxLanesLog2 = 5;
 inline int pair_lanes_log2(const CellList& cl, ab_op op) {
     const int64_t n = cl.n;
     if (op == AB_OP_SOFT && cl.g.dim == 2 && n > 1 << 15) return 0;
     const double row = (double)n / (double)cl.g.n_cells * (2 * cl.g.kx + 1);
     if (n > (1 << 18)) return 0;
-    if (row >= 100.0) return n <= 3 << 15 ? 5 : n <= 3 << 16 ? 3 : 2;
+    if (row >= 100.0) return n <= kMaxSplitN ? kMaxLanesLog2 : n <= 3 << 16 ? 3 : 2;
     if (row >= 12.0) {
         if (n <= 1 << 13) return row >= 40.0 ? 5 : 3;
         if (n <= 1 << 15) return 3;
