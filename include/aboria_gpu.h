@@ -348,10 +348,11 @@ ab_status ab_bd_step(ab_ctx* ctx, const ab_domain* dom, int64_t n,
  *           ||r||/||b|| over the columns.
  * Synchronises the context's stream before it returns, and once per iteration
  * (the stopping test) except for FP32 systems of up to 4 columns and 64 rows
- * an SM, which run in one cooperative launch with bounded waits (one that
- * gives up is reported by ab_sync as AB_ERR_TIMEOUT, W undefined).
+ * an SM, which run in one cooperative launch with bounded waits between its
+ * blocks; one that gives up makes the call return AB_ERR_TIMEOUT (W undefined,
+ * iters 0, relres infinity).
  * Errors: AB_ERR_INVALID_ARG, AB_ERR_ALIAS (W overlaps X or B),
- * AB_ERR_UNSUPPORTED, AB_ERR_OOM, AB_ERR_CUDA. */
+ * AB_ERR_UNSUPPORTED, AB_ERR_OOM, AB_ERR_CUDA, AB_ERR_TIMEOUT. */
 ab_status ab_kernel_solve(ab_ctx* ctx, int64_t n, const float* X, int32_t nrhs,
                           const float* B, float s, float sigma2, ab_prec prec,
                           float tol, int32_t max_iter, float* W, int32_t* iters,

@@ -63,6 +63,14 @@ ab_status ab_testing_build_path(ab_ctx* ctx, int32_t path);
  * one build only.  Errors: AB_ERR_INVALID_ARG. */
 ab_status ab_testing_build_timeout(ab_ctx* ctx, int32_t skip_block, int64_t limit_ns);
 
+/* Make the next ab_kernel_solve that runs in one launch exercise its bounded
+ * waits: block `skip_block` takes no part (none if the grid is smaller), so the
+ * other blocks' first wait for it gives up after `limit_ns` nanoseconds
+ * (0 < limit_ns <= 2e9) and every block returns.  Every access stays inside the
+ * library's buffers and W, the call returns AB_ERR_TIMEOUT, and the next solve
+ * is a normal one.  Errors: AB_ERR_INVALID_ARG. */
+ab_status ab_testing_solve_timeout(ab_ctx* ctx, int32_t skip_block, int64_t limit_ns);
+
 #ifdef __cplusplus
 }
 #endif

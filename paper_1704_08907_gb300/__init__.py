@@ -365,4 +365,10 @@ def ab_testing_build_timeout(ctx: Context, skip_block: int, limit_ns: int):
     _check(_lib.ab_testing_build_timeout(ctx.handle, int(skip_block), int(limit_ns)), ctx)
 
 
+def ab_testing_solve_timeout(ctx: Context, skip_block: int, limit_ns: int):
+    """Testing hook: block `skip_block` takes no part in the next one-launch
+    solve, whose waits give up after `limit_ns`."""
+    _check(_lib.ab_testing_solve_timeout(ctx.handle, int(skip_block), int(limit_ns)), ctx)
+
+
 from .autograd import GaussPairSum, KernelMatvec, LJEnergy, lj_energy_forces  # noqa: E402,F401

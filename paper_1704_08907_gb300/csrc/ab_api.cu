@@ -63,6 +63,7 @@ struct ab_ctx {
     ab::CellList cl;
     ab::Scratch sc;
     ab::BuildOptions build_opt;
+    ab::SolveWait solve_wait;   // testing: of the next one-launch solve
     int coop_launch = 0;      // the device supports cooperative launches
     int table_mode = 0;       // testing: 0 automatic, 1 dense, 2 compact where allowed
     unsigned long long dense_stream = 0;   // id of the stream that sc.dense_ws belongs to
@@ -402,8 +403,6 @@ ab_status ab_sync(ab_ctx* c) {
             return fail(c, AB_ERR_TIMEOUT, "scan look-back wait exceeded its time limit");
         if (h & ab::DEVERR_TC_TIMEOUT)
             return fail(c, AB_ERR_TIMEOUT, "tensor-core pipeline wait exceeded its time limit");
-        if (h & ab::DEVERR_SOLVE_TIMEOUT)
-            return fail(c, AB_ERR_TIMEOUT, "solve grid barrier exceeded its time limit");
     }
     return AB_OK;
 }
@@ -819,8 +818,14 @@ ab_status ab_kernel_solve(ab_ctx* c, int64_t n, const float* X, int32_t nrhs, co
         // without the memory for its slab, the stepwise form below
         e = grow(&c->sc.solve_ws, &c->sc.cap_solve_ws, ab::solve_coop_workspace_bytes(n, nrhs), c->stream);
         if (e == cudaSuccess) {
+            bool timed_out = false;
             e = ab::run_solve_coop(n, nrhs, (const float4*)X, B, s, sigma2, tol, max_iter, W,
-                                   c->sc.solve_ws, &it, &rr, c->d_err, c->stream);
+                                   c->sc.solve_ws, &it, &rr, c->solve_wait, &timed_out, c->stream);
+            c->solve_wait = ab::SolveWait{};
+            if (e == cudaSuccess && timed_out) {
+                if (relres) *relres = INFINITY;
+                return fail(c, AB_ERR_TIMEOUT, "ab_kernel_solve: a wait between blocks exceeded its time limit");
+            }
             if (e == cudaSuccess) {
                 if (iters) *iters = it;
                 if (relres) *relres = rr;
@@ -972,6 +977,13 @@ ab_status ab_testing_build_timeout(ab_ctx* c, int32_t skip_block, int64_t limit_
     if (!c || skip_block < 0 || limit_ns <= 0 || limit_ns > 2000000000ll) return AB_ERR_INVALID_ARG;
     c->build_opt.skip_block = skip_block;
     c->build_opt.limit_ns = (long long)limit_ns;
+    return AB_OK;
+}
+
+ab_status ab_testing_solve_timeout(ab_ctx* c, int32_t skip_block, int64_t limit_ns) {
+    if (!c || skip_block < 0 || limit_ns <= 0 || limit_ns > 2000000000ll) return AB_ERR_INVALID_ARG;
+    c->solve_wait.skip_block = skip_block;
+    c->solve_wait.limit_ns = (long long)limit_ns;
     return AB_OK;
 }
 

@@ -16,7 +16,6 @@ namespace ab {
 enum : uint32_t {
     DEVERR_SCAN_TIMEOUT = 1u,
     DEVERR_TC_TIMEOUT = 2u,   // a tensor-core kernel's pipeline wait gave up
-    DEVERR_SOLVE_TIMEOUT = 4u,   // a grid barrier of the one-launch solve gave up
 };
 
 // Cell-lattice geometry of one build, passed by value to kernels.
@@ -233,12 +232,18 @@ AB_HIDDEN cudaError_t run_solve(int64_t n, int nrhs, const float* B, float sigma
                                 int max_iter, float* W, void* ws, const SolveMatvec& mv,
                                 int* iters, float* relres, cudaStream_t st);
 
-// The same in one cooperative launch (FP32, few columns)
+// The same in one cooperative launch (FP32, few columns).  *timed_out: a wait
+// between its blocks ran out, and W is undefined.
+struct SolveWait {
+    int skip_block = -1;      // testing: this block takes no part
+    long long limit_ns = 0;   // 0: the default
+};
 AB_HIDDEN bool solve_coop_supported(int64_t n, int nrhs);
 AB_HIDDEN size_t solve_coop_workspace_bytes(int64_t n, int nrhs);
 AB_HIDDEN cudaError_t run_solve_coop(int64_t n, int nrhs, const float4* X, const float* B, float s,
                                      float sigma2, float tol, int max_iter, float* W, void* ws,
-                                     int* iters, float* relres, uint32_t* err, cudaStream_t st);
+                                     int* iters, float* relres, const SolveWait& wait, bool* timed_out,
+                                     cudaStream_t st);
 
 // ab_bd.cu
 AB_HIDDEN cudaError_t launch_bd_step(const Geom& g, int64_t n, float4* pos,

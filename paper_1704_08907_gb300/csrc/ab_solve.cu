@@ -243,6 +243,8 @@ constexpr long long kSolveWaitNs = 1000000000ll;
 
 struct CoopResult {
     int iters;
+    int done;        // 1 once block 0 has come to its end
+    int failed;      // 1 if a wait of any block ran out
     int pad;
     double worst;    // largest r.r / b.b
 };
@@ -265,8 +267,9 @@ struct CoopSolve {
     CoopWord* rp;              // [n][nrhs]: {r, p}; epochs 0 at launch
     CoopWord* mail;            // [2][nrhs][to][from]: partial sums; epochs 0 at launch
     float* slab;               // [blocks][n4 / 4][rows][4]
-    uint32_t* err;
     CoopResult* result;
+    long long limit_ns;        // of each wait
+    int skip_block;            // testing: this block takes no part (-1: none)
 };
 
 __device__ __forceinline__ float ex2_solve(float x) {
@@ -294,7 +297,7 @@ __device__ __forceinline__ void word_load(const CoopWord* s, uint64_t& value, ui
 // loop's exit is the warp's vote: lanes leaving one by one would leave the
 // warp split behind it (7.1 instead of 9.5 us an iteration at n = 500).
 __device__ __forceinline__ bool word_wait(const CoopWord* s, bool live, uint64_t epoch, uint64_t& value,
-                                          volatile int* dead) {
+                                          volatile int* dead, long long limit_ns) {
     long long t0 = 0;
     value = 0ull;
     for (int spin = 0;; ++spin) {
@@ -305,7 +308,7 @@ __device__ __forceinline__ bool word_wait(const CoopWord* s, bool live, uint64_t
             long long now;
             asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
             if (t0 == 0) t0 = now;
-            if (__any_sync(0xffffffffu, *dead || now - t0 > kSolveWaitNs)) {
+            if (__any_sync(0xffffffffu, *dead || now - t0 > limit_ns)) {
                 *dead = 1;
                 return false;
             }
@@ -358,6 +361,7 @@ k_solve_coop(CoopSolve a) {
     const int64_t row = i0 + lrow;
     float* slab = a.slab + (int64_t)blockIdx.x * n4 * rows;
     const int tiles = (int)((n4 + JT - 1) / JT);
+    if ((int)blockIdx.x == a.skip_block) return;
     if (t == 0) s_dead = 0;
 
     // All-reduction of one value per consumer lane and column, and a grid
@@ -387,8 +391,9 @@ k_solve_coop(CoopSolve a) {
                 for (int64_t b0 = 0; b0 < G; b0 += 32) {
                     const bool live = b0 + lane < G;
                     uint64_t w;        // a lane without a word adds 0
-                    if (!word_wait(mail + blockIdx.x * G + (live ? b0 + lane : 0), live, epoch, w, &s_dead)) {
-                        atomicOr(a.err, DEVERR_SOLVE_TIMEOUT);
+                    if (!word_wait(mail + blockIdx.x * G + (live ? b0 + lane : 0), live, epoch, w, &s_dead,
+                                   a.limit_ns)) {
+                        a.result->failed = 1;
                         break;
                     }
                     x += __longlong_as_double((long long)w);
@@ -482,8 +487,9 @@ k_solve_coop(CoopSolve a) {
             const bool live = pt < JT && j < n;
 #pragma unroll
             for (int c = 0; c < C; ++c)
-                if (!word_wait(a.rp + (live ? j * C + c : 0), live, (uint64_t)it + 1, rp[c], &s_dead))
-                    atomicOr(a.err, DEVERR_SOLVE_TIMEOUT);
+                if (!word_wait(a.rp + (live ? j * C + c : 0), live, (uint64_t)it + 1, rp[c], &s_dead,
+                               a.limit_ns))
+                    a.result->failed = 1;
         };
         auto direction = [&](int k) {      // of the points fetched last
             if (pt < JT) {
@@ -616,6 +622,7 @@ k_solve_coop(CoopSolve a) {
             for (int c = 0; c < C; ++c)
                 if (s_worst[c] > worst) worst = s_worst[c];
             a.result->iters = it;
+            a.result->done = 1;
             a.result->worst = worst;
         }
     }
@@ -693,7 +700,7 @@ size_t solve_coop_workspace_bytes(int64_t n, int nrhs) { return CoopLayout(n, nr
 // (the caller then runs run_solve).
 cudaError_t run_solve_coop(int64_t n, int nrhs, const float4* X, const float* B, float s, float sigma2,
                            float tol, int max_iter, float* W, void* ws, int* iters, float* relres,
-                           uint32_t* err, cudaStream_t st) {
+                           const SolveWait& wait, bool* timed_out, cudaStream_t st) {
     const void* fn = nrhs == 1   ? (const void*)k_solve_coop<1>
                      : nrhs == 2 ? (const void*)k_solve_coop<2>
                      : nrhs == 3 ? (const void*)k_solve_coop<3>
@@ -724,8 +731,9 @@ cudaError_t run_solve_coop(int64_t n, int nrhs, const float4* X, const float* B,
     a.rp = (CoopWord*)(q + lay.rp);
     a.mail = (CoopWord*)(q + lay.mail);
     a.slab = (float*)(q + lay.slab);
-    a.err = err;
-    // epochs start at 0; the result stays 0 if the launch gives up on a wait
+    a.limit_ns = wait.limit_ns > 0 ? wait.limit_ns : kSolveWaitNs;
+    a.skip_block = wait.skip_block;
+    // epochs start at 0, and so does the result
     if ((e = cudaMemsetAsync(q, 0, lay.clear, st)) != cudaSuccess) return e;
     void* args[] = {&a};
     e = cudaLaunchCooperativeKernel(fn, dim3((unsigned)lay.blocks), dim3(kCoopT), args, smem, st);
@@ -737,6 +745,7 @@ cudaError_t run_solve_coop(int64_t n, int nrhs, const float4* X, const float* B,
     e = cudaMemcpyAsync(&res, a.result, sizeof(res), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return e;
+    *timed_out = res.failed || !res.done;
     if (iters) *iters = res.iters;
     if (relres) *relres = (float)sqrt(res.worst);
     return cudaSuccess;
