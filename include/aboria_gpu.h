@@ -350,7 +350,9 @@ ab_status ab_bd_step(ab_ctx* ctx, const ab_domain* dom, int64_t n,
  * (the stopping test) except for FP32 systems of up to 4 columns and 64 rows
  * an SM, which run in one cooperative launch with bounded waits between its
  * blocks; one that gives up makes the call return AB_ERR_TIMEOUT (W undefined,
- * iters 0, relres infinity).
+ * iters 0, relres infinity).  That launch works on K itself, 4 n^2 bytes of
+ * device memory: up to 256 MB stay with the context, more goes back before the
+ * call returns, and where it is not to be had the other form runs.
  * Errors: AB_ERR_INVALID_ARG, AB_ERR_ALIAS (W overlaps X or B),
  * AB_ERR_UNSUPPORTED, AB_ERR_OOM, AB_ERR_CUDA, AB_ERR_TIMEOUT. */
 ab_status ab_kernel_solve(ab_ctx* ctx, int64_t n, const float* X, int32_t nrhs,

@@ -96,11 +96,13 @@ ab_status cuda_fail(ab_ctx* c, cudaError_t e, const char* where) {
 }
 
 // Stream-ordered growth: allocate the new buffer before freeing the old one,
-// so a failed allocation leaves the previous workspace intact.
+// so a failed allocation leaves the previous workspace intact.  A quarter more
+// than needed, but no more than `most` elements in all for that.
 template <typename T>
-cudaError_t grow(T** p, size_t* cap, size_t need, cudaStream_t st) {
+cudaError_t grow(T** p, size_t* cap, size_t need, cudaStream_t st, size_t most = SIZE_MAX) {
     if (need <= *cap && *p) return cudaSuccess;
     size_t want = need + need / 4 + 64;
+    if (want > most) want = need > most ? need : most;
     void* q = nullptr;
     cudaError_t e = cudaMallocAsync(&q, want * sizeof(T), st);
     if (e != cudaSuccess) {
@@ -298,6 +300,9 @@ class CallMemory {
     void* p_ = nullptr;
     bool own_ = false;
 };
+
+// One-launch solve: workspace kept between calls, at most.
+constexpr size_t kSolveKeepBytes = size_t(256) << 20;
 
 size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
 
@@ -815,13 +820,24 @@ ab_status ab_kernel_solve(ab_ctx* c, int64_t n, const float* X, int32_t nrhs, co
     int it = 0;
     float rr = 0.0f;
     if (prec == AB_PREC_FP32 && c->coop_launch && ab::solve_coop_supported(n, nrhs)) {
-        // without the memory for its slab, the stepwise form below
-        e = grow(&c->sc.solve_ws, &c->sc.cap_solve_ws, ab::solve_coop_workspace_bytes(n, nrhs), c->stream);
+        // Without the memory for its slab of K, the stepwise form below.  The
+        // context keeps slabs of up to kSolveKeepBytes (8,000 points); larger
+        // ones, up to 378 MB, go back when the call returns (2.5 us a MB).
+        const size_t need = ab::solve_coop_workspace_bytes(n, nrhs);
+        void* ws = nullptr;
+        const bool keep = need <= kSolveKeepBytes;
+        if (keep) {
+            e = grow(&c->sc.solve_ws, &c->sc.cap_solve_ws, need, c->stream, kSolveKeepBytes);
+            ws = c->sc.solve_ws;
+        } else if ((e = cudaMallocAsync(&ws, need, c->stream)) != cudaSuccess) {
+            cudaGetLastError();
+        }
         if (e == cudaSuccess) {
             bool timed_out = false;
-            e = ab::run_solve_coop(n, nrhs, (const float4*)X, B, s, sigma2, tol, max_iter, W,
-                                   c->sc.solve_ws, &it, &rr, c->solve_wait, &timed_out, c->stream);
+            e = ab::run_solve_coop(n, nrhs, (const float4*)X, B, s, sigma2, tol, max_iter, W, ws, &it, &rr,
+                                   c->solve_wait, &timed_out, c->stream);
             c->solve_wait = ab::SolveWait{};
+            if (!keep) cudaFreeAsync(ws, c->stream);
             if (e == cudaSuccess && timed_out) {
                 if (relres) *relres = INFINITY;
                 return fail(c, AB_ERR_TIMEOUT, "ab_kernel_solve: a wait between blocks exceeded its time limit");
