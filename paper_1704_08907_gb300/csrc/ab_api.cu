@@ -822,7 +822,8 @@ ab_status ab_kernel_solve(ab_ctx* c, int64_t n, const float* X, int32_t nrhs, co
     if (prec == AB_PREC_FP32 && c->coop_launch && ab::solve_coop_supported(n, nrhs)) {
         // Without the memory for its slab of K, the stepwise form below.  The
         // context keeps slabs of up to kSolveKeepBytes (8,000 points); larger
-        // ones, up to 378 MB, go back when the call returns (2.5 us a MB).
+        // ones, up to 378 MB, go back when the call returns (0.35 ms of 7.3 at
+        // 9,700 points).
         const size_t need = ab::solve_coop_workspace_bytes(n, nrhs);
         void* ws = nullptr;
         const bool keep = need <= kSolveKeepBytes;

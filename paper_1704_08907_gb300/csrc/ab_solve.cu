@@ -268,8 +268,8 @@ struct CoopSolve {
     CoopWord* mail;            // [2][nrhs][to][from]: partial sums; epochs 0 at launch
     float* slab;               // [blocks][n4 / 4][rows][4]
     CoopResult* result;
-    long long limit_ns;        // of each wait
-    int skip_block;            // testing: this block takes no part (-1: none)
+    long long limit_ns;        // testing: of each wait
+    int skip_block;            // testing: this block takes no part
 };
 
 __device__ __forceinline__ float ex2_solve(float x) {
@@ -332,7 +332,10 @@ __device__ __forceinline__ void cp_async_16(void* dst, const void* src) {
                  : "memory");
 }
 
-template <int C>
+// HOOK: the wait limit and the absent block of a test; otherwise the limit is a
+// constant, without which the poll loops took 2.4% of an iteration (n = 7,900:
+// 4.86 -> 4.98 ms).
+template <int C, bool HOOK>
 __global__ void __launch_bounds__(kCoopT, 1)
 k_solve_coop(CoopSolve a) {
     constexpr int CP = C == 3 ? 4 : C;          // columns of p in shared memory, padded
@@ -361,7 +364,8 @@ k_solve_coop(CoopSolve a) {
     const int64_t row = i0 + lrow;
     float* slab = a.slab + (int64_t)blockIdx.x * n4 * rows;
     const int tiles = (int)((n4 + JT - 1) / JT);
-    if ((int)blockIdx.x == a.skip_block) return;
+    if (HOOK && (int)blockIdx.x == a.skip_block) return;
+    const long long limit_ns = HOOK ? a.limit_ns : kSolveWaitNs;
     if (t == 0) s_dead = 0;
 
     // All-reduction of one value per consumer lane and column, and a grid
@@ -392,7 +396,7 @@ k_solve_coop(CoopSolve a) {
                     const bool live = b0 + lane < G;
                     uint64_t w;        // a lane without a word adds 0
                     if (!word_wait(mail + blockIdx.x * G + (live ? b0 + lane : 0), live, epoch, w, &s_dead,
-                                   a.limit_ns)) {
+                                   limit_ns)) {
                         a.result->failed = 1;
                         break;
                     }
@@ -488,7 +492,7 @@ k_solve_coop(CoopSolve a) {
 #pragma unroll
             for (int c = 0; c < C; ++c)
                 if (!word_wait(a.rp + (live ? j * C + c : 0), live, (uint64_t)it + 1, rp[c], &s_dead,
-                               a.limit_ns))
+                               limit_ns))
                     a.result->failed = 1;
         };
         auto direction = [&](int k) {      // of the points fetched last
@@ -701,10 +705,12 @@ size_t solve_coop_workspace_bytes(int64_t n, int nrhs) { return CoopLayout(n, nr
 cudaError_t run_solve_coop(int64_t n, int nrhs, const float4* X, const float* B, float s, float sigma2,
                            float tol, int max_iter, float* W, void* ws, int* iters, float* relres,
                            const SolveWait& wait, bool* timed_out, cudaStream_t st) {
-    const void* fn = nrhs == 1   ? (const void*)k_solve_coop<1>
-                     : nrhs == 2 ? (const void*)k_solve_coop<2>
-                     : nrhs == 3 ? (const void*)k_solve_coop<3>
-                                 : (const void*)k_solve_coop<4>;
+    const bool hook = wait.limit_ns > 0;
+    const void* fn = nrhs == 1   ? hook ? (const void*)k_solve_coop<1, true> : (const void*)k_solve_coop<1, false>
+                     : nrhs == 2 ? hook ? (const void*)k_solve_coop<2, true> : (const void*)k_solve_coop<2, false>
+                     : nrhs == 3 ? hook ? (const void*)k_solve_coop<3, true> : (const void*)k_solve_coop<3, false>
+                     : hook      ? (const void*)k_solve_coop<4, true>
+                                 : (const void*)k_solve_coop<4, false>;
     const CoopLayout lay(n, nrhs);
     if (lay.blocks > kCoopMaxBlocks) return cudaErrorNotSupported;
     CoopSolve a;
@@ -731,7 +737,7 @@ cudaError_t run_solve_coop(int64_t n, int nrhs, const float4* X, const float* B,
     a.rp = (CoopWord*)(q + lay.rp);
     a.mail = (CoopWord*)(q + lay.mail);
     a.slab = (float*)(q + lay.slab);
-    a.limit_ns = wait.limit_ns > 0 ? wait.limit_ns : kSolveWaitNs;
+    a.limit_ns = wait.limit_ns;
     a.skip_block = wait.skip_block;
     // epochs start at 0, and so does the result
     if ((e = cudaMemsetAsync(q, 0, lay.clear, st)) != cudaSuccess) return e;
