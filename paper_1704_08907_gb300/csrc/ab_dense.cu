@@ -517,11 +517,18 @@ OwnShape ordered_shape(int64_t m, int nrhs) {
 
 // Splits of the n other points: the work of a block is its points plus about
 // 64 points' worth of start and write-out, and blocks run in waves of the
-// resident ones; the number of splits with the least time in that model.
-int plan_split(int64_t blocks, int64_t n, int occ) {
+// resident ones; the number of splits with the least time in that model whose
+// partial sums (split_bytes each) take at most kMaxPartBytes.  The context keeps
+// them, and many rows gain only the last wave by them: 200,000^2 points with 64
+// columns took 12 splits and 586 MB, now 3 and 146 MB (100.0 -> 103.8 ms), 10^6
+// rows 7 and 1.7 GB for 1%, now 1.  65,536^2 keeps its 13 (208 MB, 10.9 ms).
+constexpr int64_t kMaxPartBytes = int64_t(224) << 20;
+
+int plan_split(int64_t blocks, int64_t n, int occ, int64_t split_bytes) {
     const int64_t resident = (int64_t)occ * num_sms();
     int64_t most = (n + 63) / 64;
     if (most > 256) most = 256;
+    if (split_bytes > 0 && most > kMaxPartBytes / split_bytes) most = kMaxPartBytes / split_bytes;
     int64_t best = 1, cost = INT64_MAX;
     for (int64_t s = 1; s <= most; ++s) {
         const int64_t waves = (blocks * s + resident - 1) / resident;
@@ -547,7 +554,8 @@ OwnPlan own_plan(int64_t m, int64_t n, int nrhs, bool val, bool grad, bool may_s
     const int64_t rows = (int64_t)kOwnThreads * p.sh.I;
     p.blocks = (m + rows - 1) / rows;
     p.groups = grad ? 1 : (nrhs + p.sh.R - 1) / p.sh.R;
-    p.splits = may_split ? plan_split(p.blocks * p.groups, n, p.sh.occ) : 1;
+    const int64_t split_bytes = m * ((val ? (int64_t)nrhs * 4 : 0) + (grad ? 16 : 0));
+    p.splits = may_split ? plan_split(p.blocks * p.groups, n, p.sh.occ, split_bytes) : 1;
     return p;
 }
 
