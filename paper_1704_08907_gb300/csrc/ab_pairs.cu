@@ -95,7 +95,10 @@ k_pair_fwd_q(PairParams P, PairOut o) {
             a0 *= 0.5f * P.eps;
             o.out[p] = a0;
         } else {
-            o.out4[p] = make_float4(P.fscale * a0, P.fscale * a1, DIM == 3 ? P.fscale * a2 : 0.0f, 0.0f);
+            // a sum without terms (or of coincident points alone) stays 0 also
+            // where the factor is infinite
+            auto scaled = [&](float a) { return a == 0.0f ? 0.0f : P.fscale * a; };
+            o.out4[p] = make_float4(scaled(a0), scaled(a1), DIM == 3 ? scaled(a2) : 0.0f, 0.0f);
         }
     }
     if (OP == AB_OP_LJ && o.partial) block_partial<kPairThreads>(lead ? (double)a0 : 0.0, o.partial);
