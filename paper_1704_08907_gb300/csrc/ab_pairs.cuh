@@ -26,6 +26,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <type_traits>
@@ -48,7 +49,7 @@ struct PairParams {
     int64_t n;
     Geom g;
     float s, s_log2e, eps, sig2, k, r;
-    float fscale;         // factor of a vector sum: -c (EXPF), 1 (SOFT), -20 a / r^2 (SPH force)
+    float fscale;         // factor of a vector sum: -c (EXPF), a power of two (SOFT), -20 a / r^2 (SPH force)
     float zero;   // 0.0f, passed at run time (see sq2)
     float wend_a;         // Wendland C2 normalisation a (SPH)
     float inv_r;          // 1 / r
@@ -436,6 +437,21 @@ inline PairParams make_params(const CellList& cl, ab_op op, const ab_op_params& 
     P.inv_r = (float)(1.0 / r);
     // W'(d)/d = -20 a / r^2 (1 - d/r)^3
     P.fscale = op == AB_OP_EXPF ? -prm.c : op == AB_OP_SOFT ? 1.0f : (float)(-20.0 * a / (r * r));
+    if (op == AB_OP_SOFT) {
+        // A coincident pair meets k r / FLT_MIN^(1/2) before its separation of
+        // 0.  Where that could overflow (k r > 3.7e19), a power of two is taken
+        // out of k and put back at the end, which changes no rounding.
+        const double top = fabs((double)prm.k) * (r > 1.0 ? r * r : r);
+        if (!isfinite(prm.k)) {
+            P.k = 1.0f;
+            P.fscale = prm.k;
+        } else if (top > 0x1p60) {
+            int e = ilogb(top) - 59;
+            if (e > 126) e = 126;
+            P.k = ldexpf(prm.k, -e);
+            P.fscale = ldexpf(1.0f, e);
+        }
+    }
     return P;
 }
 

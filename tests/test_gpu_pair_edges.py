@@ -38,7 +38,9 @@ def _reference(op, dim, x, r, c, k, m, A):
 
 
 CASES = [("expf", 1.0, dict(c=1.0)), ("expf", 1.0, dict(c=3e37)), ("expf", 1.0, dict(c=float("inf"))),
-         ("soft", 1.0, dict(k=1.0)),
+         ("soft", 1.0, dict(k=1.0)), ("soft", 1.0, dict(k=2e19)), ("soft", 1.0, dict(k=1e30)),
+         ("soft", 1.0, dict(k=-1e37)), ("soft", 1e12, dict(k=1e20)), ("soft", 1e-6, dict(k=1e30)),
+         ("soft", 1.0, dict(k=float("inf"))),
          ("sph_force", 1.0, dict(m=1.0, A=1.0))]
 
 
