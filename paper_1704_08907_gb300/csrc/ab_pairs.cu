@@ -63,9 +63,9 @@ k_pair_fwd_q(PairParams P, PairOut o) {
                 a0 = fmaf(sr6, sr6 - 1.0f, a0);
                 return;
             } else if (OP == AB_OP_SPH_FORCE) {
-                // m_j (A_i + A_j) (1 - d/r)^3 dx
+                // m_j (A_i + A_j) c^3 (1 - d/r)^3 dx
                 const float2 vj = DIM == 2 ? make_float2(pj.z, pj.w) : __ldg(P.sv + j);
-                const float t = fmaf(-P.inv_r, pair_distance(d2), 1.0f);
+                const float t = fmaf(-P.grad_c_inv_r, pair_distance(d2), P.grad_c);
                 mag = vj.x * (ai + vj.y) * (t * t * t);
             } else {
                 // coincident points contribute 0: a finite mag times 0

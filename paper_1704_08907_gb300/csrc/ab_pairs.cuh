@@ -49,10 +49,11 @@ struct PairParams {
     int64_t n;
     Geom g;
     float s, s_log2e, eps, sig2, k, r;
-    float fscale;         // factor of a vector sum: -c (EXPF), a power of two (SOFT), -20 a / r^2 (SPH force)
+    float fscale;         // factor of a vector sum: -c (EXPF), a power of two (SOFT), within [1, 8] (SPH force)
     float zero;   // 0.0f, passed at run time (see sq2)
     float wend_a;         // Wendland C2 normalisation a (SPH)
     float inv_r;          // 1 / r
+    float grad_c, grad_c_inv_r;   // SPH force: a power of two c, c^3 about 20 a / r^2, and c / r
 };
 
 
@@ -435,8 +436,15 @@ inline PairParams make_params(const CellList& cl, ab_op op, const ab_op_params& 
     const double a = cl.g.dim == 3 ? 21.0 / (2.0 * pi * r * r * r) : 7.0 / (pi * r * r);
     P.wend_a = (float)a;
     P.inv_r = (float)(1.0 / r);
-    // W'(d)/d = -20 a / r^2 (1 - d/r)^3
-    P.fscale = op == AB_OP_EXPF ? -prm.c : op == AB_OP_SOFT ? 1.0f : (float)(-20.0 * a / (r * r));
+    // W'(d)/d = -20 a / r^2 (1 - d/r)^3: its power of two lies within the cube, (c
+    // - c d/r)^3, which costs a pair nothing and keeps the terms in range; the rest
+    // is the sum's
+    const double f = 20.0 * a / (r * r);
+    int e = (int)floor(log2(f) / 3.0);
+    e = e < -40 ? -40 : e > 40 ? 40 : e;
+    P.grad_c = ldexpf(1.0f, e);
+    P.grad_c_inv_r = P.inv_r * P.grad_c;
+    P.fscale = op == AB_OP_EXPF ? -prm.c : op == AB_OP_SOFT ? 1.0f : (float)(-ldexp(f, -3 * e));
     if (op == AB_OP_SOFT) {
         // A coincident pair meets k r / FLT_MIN^(1/2) before its separation of
         // 0.  Where that could overflow (k r > 3.7e19), a power of two is taken
@@ -446,10 +454,10 @@ inline PairParams make_params(const CellList& cl, ab_op op, const ab_op_params& 
             P.k = 1.0f;
             P.fscale = prm.k;
         } else if (top > 0x1p60) {
-            int e = ilogb(top) - 59;
-            if (e > 126) e = 126;
-            P.k = ldexpf(prm.k, -e);
-            P.fscale = ldexpf(1.0f, e);
+            int up = ilogb(top) - 59;
+            if (up > 126) up = 126;
+            P.k = ldexpf(prm.k, -up);
+            P.fscale = ldexpf(1.0f, up);
         }
     }
     return P;

@@ -41,7 +41,8 @@ CASES = [("expf", 1.0, dict(c=1.0)), ("expf", 1.0, dict(c=3e37)), ("expf", 1.0, 
          ("soft", 1.0, dict(k=1.0)), ("soft", 1.0, dict(k=2e19)), ("soft", 1.0, dict(k=1e30)),
          ("soft", 1.0, dict(k=-1e37)), ("soft", 1e12, dict(k=1e20)), ("soft", 1e-6, dict(k=1e30)),
          ("soft", 1.0, dict(k=float("inf"))),
-         ("sph_force", 1.0, dict(m=1.0, A=1.0))]
+         ("sph_force", 1.0, dict(m=1.0, A=1.0)), ("sph_force", 1e-7, dict(m=1e-20, A=0.1)),
+         ("sph_force", 1e3, dict(m=1e35, A=50.0)), ("sph_force", 1e-6, dict(m=1e-30, A=1e-3))]
 
 
 @pytest.mark.parametrize("dim", [2, 3])
