@@ -63,6 +63,11 @@ ab_status ab_testing_build_path(ab_ctx* ctx, int32_t path);
  * one build only.  Errors: AB_ERR_INVALID_ARG. */
 ab_status ab_testing_build_timeout(ab_ctx* ctx, int32_t skip_block, int64_t limit_ns);
 
+/* What the last ab_build ran as: 0 the kernel sequence, 1 the cooperative
+ * launch, 2 the radix sort, 3 one block, 4 a cluster of 16 blocks.
+ * Errors: AB_ERR_INVALID_ARG, AB_ERR_STALE. */
+ab_status ab_testing_build_form(ab_ctx* ctx, int32_t* form);
+
 /* Make the next ab_kernel_solve that runs in one launch exercise its bounded
  * waits: block `skip_block` takes no part (none if the grid is smaller), so the
  * other blocks' first wait for it gives up after `limit_ns` nanoseconds

@@ -365,6 +365,16 @@ def ab_testing_build_timeout(ctx: Context, skip_block: int, limit_ns: int):
     _check(_lib.ab_testing_build_timeout(ctx.handle, int(skip_block), int(limit_ns)), ctx)
 
 
+FORM_SEQUENCE, FORM_COOP, FORM_RADIX, FORM_BLOCK, FORM_CLUSTER = range(5)
+
+
+def ab_testing_build_form(ctx: Context) -> int:
+    """Testing hook: what the last build ran as (FORM_...)."""
+    form = ctypes.c_int32()
+    _check(_lib.ab_testing_build_form(ctx.handle, ctypes.byref(form)), ctx)
+    return form.value
+
+
 def ab_testing_solve_timeout(ctx: Context, skip_block: int, limit_ns: int):
     """Testing hook: block `skip_block` takes no part in the next one-launch
     solve, whose waits give up after `limit_ns`."""

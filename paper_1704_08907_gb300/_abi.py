@@ -76,6 +76,7 @@ SIGNATURES = {
     "ab_testing_build_path": (ST, [P, I32]),
     "ab_testing_cell_table": (ST, [P, I32]),
     "ab_testing_build_timeout": (ST, [P, I32, I64]),
+    "ab_testing_build_form": (ST, [P, P]),
     "ab_testing_solve_timeout": (ST, [P, I32, I64]),
     "ab_exclusive_scan_u32_static": (ST, [P, P, I64, P]),
 }

@@ -997,6 +997,14 @@ ab_status ab_testing_build_timeout(ab_ctx* c, int32_t skip_block, int64_t limit_
     return AB_OK;
 }
 
+ab_status ab_testing_build_form(ab_ctx* c, int32_t* form) {
+    if (!c || !form) return AB_ERR_INVALID_ARG;
+    ab_status s = require_cells(c);
+    if (s != AB_OK) return s;
+    *form = c->cl.form;
+    return AB_OK;
+}
+
 ab_status ab_testing_solve_timeout(ab_ctx* c, int32_t skip_block, int64_t limit_ns) {
     if (!c || skip_block < 0 || limit_ns <= 0 || limit_ns > 2000000000ll) return AB_ERR_INVALID_ARG;
     c->solve_wait.skip_block = skip_block;

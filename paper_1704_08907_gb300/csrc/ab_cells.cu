@@ -1163,6 +1163,7 @@ cudaError_t launch_build(CellList& cl, const float* pos, bool packed, Scratch& s
     // 56.4 us; 4M points in 2-D 176.8 vs 167.6 us).
     constexpr int64_t kSingleLaunchMaxN = int64_t(1) << 21;
     const int path = opt.path == kPathAuto ? auto_build_path(n, cl.g) : opt.path;
+    cl.form = kFormRadix;
     if (path == kPathRadix && radix_supported(n, nc))
         return launch_build_radix(cl, pos, packed, sc, err, st, opt);
     if (!compact && opt.path == kPathAuto && opt.skip_block < 0 && n > kClusterMinN && n <= kClusterMaxN &&
@@ -1178,6 +1179,7 @@ cudaError_t launch_build(CellList& cl, const float* pos, bool packed, Scratch& s
         a.spos = cl.spos;
         const cudaError_t e = cl.g.dim == 3 ? (packed ? launch_cluster<3, true>(a, st) : launch_cluster<3, false>(a, st))
                                             : (packed ? launch_cluster<2, true>(a, st) : launch_cluster<2, false>(a, st));
+        cl.form = kFormCluster;
         if (e == cudaSuccess) return e;
         cudaGetLastError();   // no room for the cluster on this device: the forms below
     }
@@ -1191,6 +1193,7 @@ cudaError_t launch_build(CellList& cl, const float* pos, bool packed, Scratch& s
         a.cell_start = cl.cell_start;
         a.perm = cl.perm;
         a.spos = cl.spos;
+        cl.form = kFormBlock;
         if (cl.g.dim == 3) return packed ? launch_small<3, true>(a, st) : launch_small<3, false>(a, st);
         return packed ? launch_small<2, true>(a, st) : launch_small<2, false>(a, st);
     }
@@ -1224,6 +1227,7 @@ cudaError_t launch_build(CellList& cl, const float* pos, bool packed, Scratch& s
             a.limit_ns = opt.limit_ns > 0 ? opt.limit_ns : kScanLimitNs;
             a.skip_block = opt.skip_block < grid ? opt.skip_block : -1;
             void* args[] = {&a};
+            cl.form = kFormCoop;
             cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3((unsigned)grid), dim3(kCoopThreads), args, 0, st);
             if (e == cudaSuccess || compact) return e;
             cudaGetLastError();   // not launchable here: fall back to the kernel sequence
@@ -1231,6 +1235,7 @@ cudaError_t launch_build(CellList& cl, const float* pos, bool packed, Scratch& s
         if (compact) return cudaErrorNotSupported;
     }
     if (compact) return cudaErrorNotSupported;
+    cl.form = kFormSequence;
     cudaError_t e = cudaMemsetAsync(cl.cell_start, 0, (size_t)(nc + 1) * sizeof(uint32_t), st);
     if (e != cudaSuccess) return e;
     if (n > 0) {

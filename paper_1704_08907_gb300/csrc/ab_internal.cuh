@@ -62,6 +62,7 @@ struct CellList {
     // 32-63) and the number of occupied cells before them (z)
     uint4* occ = nullptr;
     size_t cap_occ = 0;
+    int form = 0;                     // BuildForm of the last build
 };
 
 // Words of the occupancy table of a compact cell list (cells 0 .. n_cells,
@@ -98,6 +99,8 @@ struct Scratch {
 // sort of ab_sort.cu, or the automatic choice; the last two fields are
 // testing hooks of the bounded waits.
 enum BuildPath : int { kPathSequence = 0, kPathCoop = 1, kPathRadix = 2, kPathAuto = 3 };
+// What a build ran as.
+enum BuildForm : int { kFormSequence = 0, kFormCoop = 1, kFormRadix = 2, kFormBlock = 3, kFormCluster = 4 };
 struct BuildOptions {
     int path = kPathAuto;
     int skip_block = -1;          // a block (tile) that never arrives (publishes)
