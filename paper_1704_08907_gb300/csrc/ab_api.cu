@@ -373,6 +373,10 @@ ab_status ab_destroy(ab_ctx* c) {
     if (!c) return AB_OK;
     ab::DeviceGuard dg(c->device);
     cudaStreamSynchronize(c->stream);
+    // dense calls may have run on another stream than the last one set
+    unsigned long long id = 0;
+    if (c->sc.dense_ws && (cudaStreamGetId(c->stream, &id) != cudaSuccess || id != c->dense_stream))
+        cudaDeviceSynchronize();
     void* bufs[] = {c->cl.spos, c->cl.perm, c->cl.cell_rank, c->cl.tmp,
                     c->cl.cell_start, c->cl.occ, c->sc.sv, c->sc.scan_status, c->sc.scan_ticket,
                     c->sc.partial, c->sc.counts, c->sc.dense_ws, c->sc.solve_ws, c->sc.coop,

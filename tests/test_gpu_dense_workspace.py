@@ -115,3 +115,27 @@ def test_memory_is_given_back(ab, cuda):
     held, after = used()
     assert before - held <= 256 << 20       # the 138 MB of partial sums, a quarter more, the cell list's own
     assert before - after <= 32 << 20
+
+
+def test_destroyed_while_the_first_stream_runs(ab, cuda):
+    """The buffer belongs to the stream of the first dense call; the context is
+    destroyed on another one while that stream is still at work."""
+    m, n = 4000, 60000
+    X, Y, W, _ = _inputs(m, n, 64, 6)
+    ctx = ab.Context(0)
+    want = ab.ab_kernel_matvec(ctx, X, Y, W, S, "fp32")
+    ctx.close()
+    got = [torch.zeros_like(want) for _ in range(20)]
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    ctx = ab.Context(0)
+    with torch.cuda.stream(side):
+        for g in got:
+            ab.ab_kernel_matvec(ctx, X, Y, W, S, "fp32", out=g)
+    ab.ab_kernel_matvec(ctx, X[:10], Y[:10], W[:10], S, "fp32")
+    ctx.close()
+    other = ab.Context(0)
+    last = ab.ab_kernel_matvec(other, X, Y, W, S, "fp32")
+    torch.cuda.synchronize()
+    assert torch.equal(last, want) and all(torch.equal(g, want) for g in got)
+    other.close()
