@@ -8,8 +8,9 @@ namespace {
 
 // Forward for the cheap operators (COUNT, GAUSS, SPH density): direct visit.
 // The weight w_j (GAUSS) or mass m_j (SPH) comes in the pad component of the
-// sorted position, loaded with the candidate.
-template <int DIM, int MODE, int SL, int OP>
+// sorted position, loaded with the candidate.  RARE (SPH): few candidates are
+// neighbours (see visit_pairs).
+template <int DIM, int MODE, int SL, int OP, bool RARE = false>
 __global__ void __launch_bounds__(kPairThreads, 8)
 k_pair_fwd(PairParams P, PairOut o) {
     wait_prerequisite();
@@ -27,7 +28,7 @@ k_pair_fwd(PairParams P, PairOut o) {
                 a0 = fmaf(pj.w, ex2_approx(-P.s_log2e * d2), a0);
             } else {   // SPH_DENSITY: m_j W(d) / a
                 // (1 - q)^4 (1 + 4 q), q = d / r, in t = 1 - q
-                const float t = fmaf(-P.inv_r, pair_distance(d2), 1.0f), t2 = t * t;
+                const float t = fmaf(-P.inv_r, pair_distance<RARE>(d2), 1.0f), t2 = t * t;
                 a0 = fmaf(pj.w, t2 * t2 * fmaf(-4.0f, t, 5.0f), a0);
             }
         });
@@ -37,8 +38,9 @@ k_pair_fwd(PairParams P, PairOut o) {
     o.out[__ldg(P.perm + s)] = a0;
 }
 
-// Forward for LJ / EXPF / SOFT: direct visit.
-template <int DIM, int MODE, int SL, int OP>
+// Forward for LJ / EXPF / SOFT / SPH force: direct visit.  RARE (SPH force): few
+// candidates are neighbours (see visit_pairs).
+template <int DIM, int MODE, int SL, int OP, bool RARE = false>
 __global__ void __launch_bounds__(kPairThreads, 8)
 k_pair_fwd_q(PairParams P, PairOut o) {
     allow_dependents();
@@ -49,7 +51,7 @@ k_pair_fwd_q(PairParams P, PairOut o) {
     const float4 pi = live ? __ldg(P.spos + s) : make_float4(0.f, 0.f, 0.f, 0.f);
     float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f;
     const float ai = OP != AB_OP_SPH_FORCE ? 0.0f : DIM == 2 ? pi.w : live ? __ldg(&P.sv[s].y) : 0.0f;
-    if (live) visit_pairs<DIM, MODE, (OP == AB_OP_EXPF || OP == AB_OP_SOFT) ? 4 : 2, SL>(P, s, sub, pi,
+    if (live) visit_pairs<DIM, MODE, (OP == AB_OP_EXPF || OP == AB_OP_SOFT || RARE) ? 4 : 2, SL>(P, s, sub, pi,
         [&](uint32_t j, const float4& pj, float dx, float dy, float dz, float d2) {
             // EXPF and the SPH force leave out their common factor P.fscale
             // (one multiplication a particle instead of one a pair; SOFT
@@ -65,7 +67,7 @@ k_pair_fwd_q(PairParams P, PairOut o) {
             } else if (OP == AB_OP_SPH_FORCE) {
                 // m_j (A_i + A_j) c^3 (1 - d/r)^3 dx
                 const float2 vj = DIM == 2 ? make_float2(pj.z, pj.w) : __ldg(P.sv + j);
-                const float t = fmaf(-P.grad_c_inv_r, pair_distance(d2), P.grad_c);
+                const float t = fmaf(-P.grad_c_inv_r, pair_distance<RARE>(d2), P.grad_c);
                 mag = vj.x * (ai + vj.y) * (t * t * t);
             } else {
                 // coincident points contribute 0: a finite mag times 0
@@ -155,8 +157,12 @@ cudaError_t launch_pair_fwd(const CellList& cl, ab_op op, const ab_op_params& pr
         case AB_OP_LJ: return AB_PAIR_LAUNCH(k_pair_fwd_q<DIM, MODE, SL, AB_OP_LJ>);
         case AB_OP_EXPF: return AB_PAIR_LAUNCH(k_pair_fwd_q<DIM, MODE, SL, AB_OP_EXPF>);
         case AB_OP_SOFT: return AB_PAIR_LAUNCH(k_pair_fwd_q<DIM, MODE, SL, AB_OP_SOFT>);
-        case AB_OP_SPH_DENSITY: return AB_PAIR_LAUNCH(k_pair_fwd<DIM, MODE, SL, AB_OP_SPH_DENSITY>);
-        case AB_OP_SPH_FORCE: return AB_PAIR_LAUNCH(k_pair_fwd_q<DIM, MODE, SL, AB_OP_SPH_FORCE>);
+        case AB_OP_SPH_DENSITY:
+            if (pairs_are_rare(cl)) return AB_PAIR_LAUNCH(k_pair_fwd<DIM, MODE, SL, AB_OP_SPH_DENSITY, DIM == 3>);
+            return AB_PAIR_LAUNCH(k_pair_fwd<DIM, MODE, SL, AB_OP_SPH_DENSITY>);
+        case AB_OP_SPH_FORCE:
+            if (pairs_are_rare(cl)) return AB_PAIR_LAUNCH(k_pair_fwd_q<DIM, MODE, SL, AB_OP_SPH_FORCE, DIM == 3>);
+            return AB_PAIR_LAUNCH(k_pair_fwd_q<DIM, MODE, SL, AB_OP_SPH_FORCE>);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -72,9 +72,14 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-// Distance of a pair at d^2, 0 for coincident points (the floor keeps the
-// reciprocal root finite; one operation where a test and a select took two).
+// Distance of a pair at d^2, 0 for coincident points: with a floor that keeps
+// the reciprocal root finite, one operation where a test and a select take two,
+// or (BRANCH) with the test, beside which the compiler leaves the body behind a
+// branch instead of issuing it under a predicate on every candidate.  The same
+// bits.
+template <bool BRANCH>
 __device__ __forceinline__ float pair_distance(float d2) {
+    if (BRANCH) return d2 > 0.0f ? d2 * rsqrt_approx(d2) : 0.0f;
     return d2 * rsqrt_approx(fmaxf(d2, 1.17549435e-38f));
 }
 
@@ -278,6 +283,18 @@ __device__ __forceinline__ float pred_d2(const Geom& g, const float4& pi, const 
 // more FP32 ones: 417.  With its factor k taken out of the sum too: 381, 331
 // and 4,886, not kept because it changes the last bits, see pair_lanes_log2.)
 //
+// Where few candidates are neighbours (cells wider than the cut-off, as when the
+// table of a sparse or clustered input reaches its size limit: 2.6% of a stencil
+// twice as wide, 21% else) the SPH bodies are better left behind a branch (see
+// pair_distance), and the SPH force then unrolled by 4.  us, floor / branch (SPH
+// force: and 4), 3-D points:
+//   stencil 162 r^3  1M in 250 blobs  density 705 / 664   force 832 / 648
+//                    250,000 in 62            257 / 246         297 / 249
+//   stencil 20 r^3   16.7M in 1,024         5,090 / 5,046     6,050 / 6,500
+//                    1M on a lattice          333 / 336         386 / 413
+//   2-D              1M on a lattice          104 / 107         107 / 115
+// so they branch where the stencil is larger than kRareStencil r^3.
+//
 // Direct visit: f(j, pj, dx, dy, dz, d2) for every accepted pair, with value
 // separations accurate to one rounding (see value_sep).  Used by every pair
 // kernel.  UNROLL is the unroll factor of the candidate loop, measured per
@@ -373,6 +390,19 @@ __device__ __forceinline__ void block_partial(double v, double* partial) {
         for (int w = 0; w < THREADS / 32; ++w) t += s_red[w];
         partial[blockIdx.x] = t;
     }
+}
+
+// Volume of the stencil over r^3 in 3-D above which a pair is rare.
+constexpr double kRareStencil = 70.0;
+inline bool pairs_are_rare(const CellList& cl) {
+    if (cl.g.dim != 3) return false;
+    const int reach[3] = {cl.g.kx, cl.g.ky, cl.g.kz};
+    double v = 1.0;
+    for (int k = 0; k < 3; ++k) {
+        const int cells = 2 * reach[k] + 1 < cl.g.n[k] ? 2 * reach[k] + 1 : cl.g.n[k];
+        v *= (double)cells / cl.g.n[k] * cl.g.L[k] / cl.g.r;
+    }
+    return v > kRareStencil;
 }
 
 // Lanes that share a particle's walk (log2), the same for every table of a
