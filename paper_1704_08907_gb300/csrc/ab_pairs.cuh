@@ -406,7 +406,9 @@ inline bool pairs_are_rare(const CellList& cl) {
 }
 
 // Lanes that share a particle's walk (log2), the same for every table of a
-// cell list and, but for SOFT in 2-D, for every operator, so that their
+// cell list and, but for SOFT in 2-D and counts (exact in any order: 250,000
+// points with 600 neighbours 192 us with four lanes, 176 with one), for every
+// operator, so that their
 // results can be compared bit for bit.  SOFT drives time steppers in place: a
 // last bit of a force moves a position by one, and a pair closer than some
 // 30,000 of them then turns by more than a thousandth in the next step.
@@ -435,6 +437,7 @@ constexpr int kMaxLanesLog2 = 5;
 inline int pair_lanes_log2(const CellList& cl, ab_op op) {
     const int64_t n = cl.n;
     if (op == AB_OP_SOFT && cl.g.dim == 2 && n > 1 << 15) return 0;
+    if (op == AB_OP_COUNT && n > 3 << 16) return 0;
     const double row = (double)n / (double)cl.g.n_cells * (2 * cl.g.kx + 1);
     if (n > (1 << 18)) return 0;
     if (row >= 100.0) return n <= kMaxSplitN ? kMaxLanesLog2 : n <= 3 << 16 ? 3 : 2;
