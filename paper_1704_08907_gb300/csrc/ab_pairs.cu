@@ -158,10 +158,10 @@ cudaError_t launch_pair_fwd(const CellList& cl, ab_op op, const ab_op_params& pr
         case AB_OP_EXPF: return AB_PAIR_LAUNCH(k_pair_fwd_q<DIM, MODE, SL, AB_OP_EXPF>);
         case AB_OP_SOFT: return AB_PAIR_LAUNCH(k_pair_fwd_q<DIM, MODE, SL, AB_OP_SOFT>);
         case AB_OP_SPH_DENSITY:
-            if (pairs_are_rare(cl)) return AB_PAIR_LAUNCH(k_pair_fwd<DIM, MODE, SL, AB_OP_SPH_DENSITY, DIM == 3>);
+            if (pairs_are_rare(cl)) return AB_PAIR_LAUNCH(k_pair_fwd<DIM, MODE, SL, AB_OP_SPH_DENSITY, DIM == 3 && SL == 0>);
             return AB_PAIR_LAUNCH(k_pair_fwd<DIM, MODE, SL, AB_OP_SPH_DENSITY>);
         case AB_OP_SPH_FORCE:
-            if (pairs_are_rare(cl)) return AB_PAIR_LAUNCH(k_pair_fwd_q<DIM, MODE, SL, AB_OP_SPH_FORCE, DIM == 3>);
+            if (pairs_are_rare(cl)) return AB_PAIR_LAUNCH(k_pair_fwd_q<DIM, MODE, SL, AB_OP_SPH_FORCE, DIM == 3 && SL == 0>);
             return AB_PAIR_LAUNCH(k_pair_fwd_q<DIM, MODE, SL, AB_OP_SPH_FORCE>);
         default: return cudaErrorInvalidValue;
     }

@@ -293,7 +293,8 @@ __device__ __forceinline__ float pred_d2(const Geom& g, const float4& pi, const 
 //   stencil 20 r^3   16.7M in 1,024         5,090 / 5,046     6,050 / 6,500
 //                    1M on a lattice          333 / 336         386 / 413
 //   2-D              1M on a lattice          104 / 107         107 / 115
-// so they branch where the stencil is larger than kRareStencil r^3.
+// so they branch where the stencil is larger than kRareStencil r^3 and a particle
+// has one lane (with four, 50,000 points of which many crowd: force 65 / 85).
 //
 // Direct visit: f(j, pj, dx, dy, dz, d2) for every accepted pair, with value
 // separations accurate to one rounding (see value_sep).  Used by every pair
@@ -406,29 +407,35 @@ inline bool pairs_are_rare(const CellList& cl) {
 }
 
 // Lanes that share a particle's walk (log2), the same for every table of a
-// cell list and, but for SOFT in 2-D and counts (exact in any order: 250,000
-// points with 600 neighbours 192 us with four lanes, 176 with one), for every
-// operator, so that their
-// results can be compared bit for bit.  SOFT drives time steppers in place: a
-// last bit of a force moves a position by one, and a pair closer than some
-// 30,000 of them then turns by more than a thousandth in the next step.
-// Points in the plane come that close by chance from about a hundred thousand
-// of them, so there SOFT keeps one lane and the order of its sums.
+// cell list and, but for SOFT and counts (exact in any order) in 2-D, for every
+// operator, so that their results can be compared bit for bit.  SOFT drives
+// time steppers in place: a last bit of a force moves a position by one, and a
+// pair closer than some 30,000 of them then turns by more than a thousandth in
+// the next step.  Points in the plane come that close by chance from about a
+// hundred thousand of them, so there SOFT keeps one lane and the order of its
+// sums.
 // One lane a particle while the particles fill the SMs.  Fewer leave SMs
 // idle, and one lane's walk, thousands of dependent loads on dense inputs, is
 // all there is to wait for; more lanes then share it, but each row of a
 // stencil costs a lane its set-up and a warp its longest lane, so short rows
-// take fewer.  row: candidates expected in a stencil row.  Measured, us with
-// 1 / 2 / 4 / 8 / 32 lanes (EXPF; the other operators alike):
-//   row 7:    1,000  9.3/ 8.2/ 6.6/ 5.0/ 4.6    32,768  11.2/ 8.8/ 7.8/ 8.2/ 21
-//            65,536 10.9/ 9.8/ 9.9/ 12 / 36    131,072  12.8/13.0/14.4/21.1/ 69
-//   row 18:  16,384   64/  48/  27/  19/  32    65,536    65/  46/  38/  42/ 98
-//           100,003   74/  58/  48/  59/ 145   200,000    87/  80/  79/ 104/328
-//           262,144  102/  92/  98/ 134/ 362   400,000   124/ 125/ 141/ 197/646
-//   row 55:   4,096   39/  29/  15/  10/ 6.0    32,768    36/  27/  18/  15/ 26
-//           200,000   53/  50/  44/  51/ 137
-//   row 215+: 65,536 512/ 366/ 261/ 204/ 181   131,072   264/ 236/ 184/ 164/184
-//           262,144  183/ 178/ 159/ 162/ 286   524,288   291/ 304/ 292/ 304/570
+// take fewer.  row: candidates expected in a stencil row.  Time over the best
+// of the five, 1 / 2 / 4 / 8 / 32 lanes (geometric mean of EXPF, counts,
+// Gaussian adjoint and fused LJ in 2-D and 3-D, uniform points):
+//   row 1:    16,384 1.21/1.10/1.01/1.06/2.1    65,536 1.09/1.01/1.33/1.85/5.2
+//   row 8:    16,384 1.83/1.33/1.07/1.00/1.9    65,536 1.26/1.02/1.10/1.32/3.8
+//            120,000 1.06/1.03/1.16/1.56/5.0   196,608 1.03/1.08/1.35/1.93/6.7
+//   row 25:   32,768 2.29/1.59/1.03/1.14/2.2    98,304 1.45/1.10/1.00/1.26/3.4
+//            196,608 1.12/1.01/1.04/1.39/4.1   262,144 1.07/1.01/1.10/1.51/4.6
+//   row 60:    8,192 3.84/2.45/1.47/1.05/1.04  196,608 1.18/1.08/1.01/1.16/2.8
+//   row 130:  12,000 4.63/2.95/1.78/1.08/1.00   16,384 4.29/2.71/1.55/1.00/1.2
+//             98,304 1.70/1.29/1.04/1.01/1.75  230,000 1.18/1.09/1.01/1.06/2.1
+//   row 260:  16,384 5.74/3.76/2.11/1.21/1.00   65,536 2.18/1.58/1.24/1.00/1.2
+//   row 500:  50,000 2.82/2.08/1.33/1.06/1.00  160,000 1.45/1.33/1.09/1.00/1.2
+//   row 1000: 80,000 2.27/1.75/1.42/1.13/1.00
+// Rows that are short on average may be long where points crowd, so up to
+// 65,536 particles they keep more lanes than uniform points want: 50,000 points,
+// a fiftieth of them at one place, density 48 us with four lanes and 173 with
+// one, 65,536 uniform points with half a neighbour 27 and 19.
 // Million-particle inputs lose 10-20% with two lanes already.
 // No rule gives more than kMaxSplitN << kMaxLanesLog2 lanes in all, or a
 // particle more than 2^kMaxLanesLog2 (pair_partial_capacity builds on it).
@@ -437,10 +444,15 @@ constexpr int kMaxLanesLog2 = 5;
 inline int pair_lanes_log2(const CellList& cl, ab_op op) {
     const int64_t n = cl.n;
     if (op == AB_OP_SOFT && cl.g.dim == 2 && n > 1 << 15) return 0;
-    if (op == AB_OP_COUNT && n > 3 << 16) return 0;
+    // counts have the shortest body: 250,000 points in 2-D with 600 neighbours 192
+    // us with four lanes, 176 with one (3-D, 340: 299 and 373)
+    if (op == AB_OP_COUNT && cl.g.dim == 2 && n > 3 << 16) return 0;
     const double row = (double)n / (double)cl.g.n_cells * (2 * cl.g.kx + 1);
     if (n > (1 << 18)) return 0;
-    if (row >= 100.0) return n <= kMaxSplitN ? kMaxLanesLog2 : n <= 3 << 16 ? 3 : 2;
+    if (row >= 100.0) {
+        if (n <= kMaxSplitN && (double)n <= 125.0 * row) return kMaxLanesLog2;
+        return n <= 3 << 16 ? 3 : 2;
+    }
     if (row >= 12.0) {
         if (n <= 1 << 13) return row >= 40.0 ? 5 : 3;
         if (n <= 1 << 15) return 3;
