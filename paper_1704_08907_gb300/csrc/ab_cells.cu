@@ -1086,10 +1086,14 @@ int auto_build_path(int64_t n, const Geom& g) {
 }
 
 // Particles and shared memory (offsets and slots) up to which the one-block
-// build is taken where the cluster's is not (8,192 points: 16 us against the
-// cooperative form's 21).
+// build is taken where the cluster's is not, unless its one SM would compare too
+// many members for their stable ranks (n^2 / cells of them; one block /
+// cooperative form, us: 2,000 points in one cell 35 / 41, 3,000 with 187 a cell
+// 27 / 27, 5,000 with 34 19 / 21, 4,096 with 256 45 / 31, 6,000 with 41 23 / 21,
+// with 666 146 / 51).
 constexpr int64_t kSmallMaxN = 8192;
 constexpr size_t kSmallMaxSmem = 128 * 1024;
+constexpr int64_t kSmallAnyN = 2048, kSmallMembers = 240000;
 
 static size_t small_smem(int64_t n, int64_t nc1) {
     return (size_t)(((nc1 + 3) & ~(int64_t)3) + n) * sizeof(uint32_t);
@@ -1184,7 +1188,7 @@ cudaError_t launch_build(CellList& cl, const float* pos, bool packed, Scratch& s
         cudaGetLastError();   // no room for the cluster on this device: the forms below
     }
     if (!compact && opt.path == kPathAuto && opt.skip_block < 0 && n <= kSmallMaxN &&
-        small_smem(n, nc + 1) <= kSmallMaxSmem) {
+        (n <= kSmallAnyN || n * n <= kSmallMembers * nc) && small_smem(n, nc + 1) <= kSmallMaxSmem) {
         CoopArgs a = {};
         a.pos = pos;
         a.n = n;

@@ -49,11 +49,13 @@ def test_form_and_list(cuda, dim, n, cells, crowded, form, packed):
     ctx.close()
 
 
-# 2 x rows cells, periodic: 32 particles a cell is the cluster's limit, past it one
-# block's (up to 8,192) or the cooperative launch; 195 table entries, 13 a
-# block, leave the cluster's last block without any
+# 2 x rows cells, periodic: 32 particles a cell is the cluster's limit, past it
+# one block or the cooperative launch, which also takes over from one block
+# above 2,048 particles at n^2 = 240,000 cells; 195 table entries, 13 a block,
+# leave the cluster's last block without any
 @pytest.mark.parametrize("rows,n,form", [(97, 6208, CLUSTER), (97, 6209, BLOCK), (128, 8192, CLUSTER),
-                                         (127, 8192, BLOCK), (200, 12800, CLUSTER), (200, 12801, COOP)])
+                                         (1, 2048, BLOCK), (4, 2049, COOP), (30, 3790, BLOCK),
+                                         (30, 3796, COOP), (127, 8192, COOP), (200, 12800, CLUSTER), (200, 12801, COOP)])
 def test_particles_a_cell(cuda, rows, n, form):
     import paper_1704_08907_gb300 as ab
     r = 0.125
