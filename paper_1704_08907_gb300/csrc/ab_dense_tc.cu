@@ -1487,10 +1487,11 @@ int fwd_splits(ab_prec prec, int64_t m, int64_t n, bool ordered) {
 // chain a thread: their ranges too are never longer than those of two ranges for
 // fewer than four waves of row blocks (19,456 rows x 30,000 points, one wave:
 // terms of one sign: one range 289 us and off by 2.6e-7 of the sum, rms, two 298
-// us and 1.8e-7).
+// us and 1.8e-7).  Up to 2,048 points one range is no further off than two
+// (1.86e-7 and 1.87e-7), and two cost a launch more, 2.5 us of the host's time.
 int grad_splits(int64_t m, int64_t n) {
     const int64_t mblocks = (m + 127) / 128, tiles = (n + 127) / 128;
-    const int least = mblocks < 4 * (int64_t)num_sms() && tiles >= 2 ? 2 : 1;
+    const int least = mblocks < 4 * (int64_t)num_sms() && tiles > 16 ? 2 : 1;
     return tc_splits(mblocks, tiles, 16, least, 32);
 }
 
