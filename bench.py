@@ -54,8 +54,8 @@ OPS_PER_PAIR_LJ_EG = 12
 # DRAM traffic of one k_pair_lj_eg<3,false> launch on this workload, from an
 # ncu --set full capture (dram__bytes_read.sum + dram__bytes_write.sum), valid
 # only for the kernel source it was taken on (None until captured).
-TRAFFIC_EG_BYTES = 35.45e6   # 29.22 MB read + 6.23 MB written
-TRAFFIC_SOURCE_SHA = "86c1f0575ff170b2"
+TRAFFIC_EG_BYTES = 35.43e6   # 29.21 MB read + 6.22 MB written
+TRAFFIC_SOURCE_SHA = "bd8ca8df0491cd90"
 
 
 def pair_source_sha():
@@ -610,9 +610,9 @@ def oracle_sample_c3(w, nq, seed=23):
 # DRAM traffic of one k_pair_bwd<3,false,GAUSS> launch on the clustered
 # workload (ncu dram__bytes_read.sum + dram__bytes_write.sum), valid for the
 # kernel source whose hash is given (None until captured on that source).
-TRAFFIC_C3_BWD_BYTES = 942.08e6    # 549.40 MB read + 392.68 MB written (adjoint kernel)
-TRAFFIC_C3_VG_BYTES = 1129.62e6    # 612.22 MB read + 517.40 MB written (value and gradient)
-TRAFFIC_C3_SOURCE_SHA = "86c1f0575ff170b2"
+TRAFFIC_C3_BWD_BYTES = 942.84e6    # 549.89 MB read + 392.95 MB written (adjoint kernel)
+TRAFFIC_C3_VG_BYTES = 1129.34e6    # 612.16 MB read + 517.18 MB written (value and gradient)
+TRAFFIC_C3_SOURCE_SHA = "bd8ca8df0491cd90"
 
 
 def also_c3(reps=5, oracle_fraction=64):

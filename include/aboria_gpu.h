@@ -38,7 +38,8 @@
  *    (the device's default memory pool); AB_ERR_OOM leaves the context
  *    usable with its previous workspace.  The dense calls (ab_kernel_matvec
  *    and its adjoint) share no workspace between streams, and captured in a
- *    graph they use an allocation of the graph's own.
+ *    graph they use an allocation of the graph's own; the FP32 ones keep up
+ *    to 224 MB of partial sums (and the quarter more that buffers grow by).
  *  - Each call makes the context's device current while it runs and
  *    restores the caller's current device before it returns; a failure to
  *    select the device returns AB_ERR_CUDA.
@@ -152,9 +153,12 @@ ab_status ab_sync(ab_ctx* ctx);
  * empty), the library keeps offsets of the occupied cells only, with a
  * bitmap of occupied cells to find them (about 0.25 bytes a cell plus 4 a
  * particle instead of 4 bytes a cell); the order and every result are the
- * same bit for bit.  Few particles (8,192, and tables that fit shared memory
- * beside them) are built by one block, up to 16,384 by a cluster of 16.  Up to 2^21 particles, and for every
- * compact table, the build runs as one cooperative launch whose phases are separated by grid
+ * same bit for bit.  Up to 6,144 particles whose table fits shared memory
+ * beside them are built by one block, up to 16,384 and 32 a cell by a cluster
+ * of 16 (up to 8,192 by one block where the cluster is not taken; above 2,048
+ * particles with crowded cells by neither).  Up to 2^21 particles otherwise,
+ * and for every compact table, the build runs as one cooperative launch whose
+ * phases are separated by grid
  * barriers with bounded waits (a wait that gives up is reported by ab_sync
  * as AB_ERR_TIMEOUT); larger dense builds run as a sequence of kernels.
  *   dom:  host pointer to the domain (copied).

@@ -211,8 +211,8 @@ AB_HIDDEN cudaError_t launch_dense_combine(int splits, int64_t vals, const float
                                            int64_t grads, const float4* pg, float4* grad,
                                            cudaStream_t st);
 
-// ab_dense_tc.cu (tcgen05 path; nrhs must be 64).  ordered: the sums' order
-// does not depend on m (the solve)
+// ab_dense_tc.cu (tcgen05 path; nrhs must be 64).  ordered: one or two ranges
+// of points by the row blocks alone (the solve)
 AB_HIDDEN size_t dense_tc_workspace_bytes(int64_t m, int64_t n, ab_prec prec, bool ordered);
 AB_HIDDEN cudaError_t launch_dense_tc_fwd(int64_t m, int64_t n, const float4* X, const float4* Y,
                                           int nrhs, const float* W, float s, ab_prec prec,

@@ -226,7 +226,7 @@ k_solve_finish(const double* __restrict__ partial, int blocks, int nrhs, int wha
 // Bound: the chain's latency (n = 4096: 16,384 clocks, 8.4 us an iteration)
 // and the two reductions.  The form it replaces launched seven kernels an
 // iteration on 16-32 blocks, padded one column to 64 and waited on the host
-// each time.  n = 4096, one column, tol 1e-4, 64 iterations: 32.4 ms ->
+// each time.  n = 4096, one column, tol 1e-4, 69 iterations: 32.4 ms ->
 // 1.57 ms, W and the iteration count bit for bit.  Of an iteration's 22.7
 // us the chains take 17.5: 8.3 clocks a point beside the slab's copies (6.6
 // without them, 5.1 with nothing else on the SM).  Measured on the way: K

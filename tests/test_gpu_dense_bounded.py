@@ -1,6 +1,6 @@
 """Partial sums of the FP32 dense walk: what a context holds after a product
 and an adjoint of many rows stays within the bound (224 MB and the quarter that
-buffers grow by; 64 MB more for the driver's granularity), and rows and points
+buffers grow by; 64 MB more for the allocator's granularity), and rows and points
 on both sides of the bound agree with FP64 (GPU, C ABI; metric and 1e-5 of
 tests/test_gpu_dense.py on sampled rows)."""
 import pytest

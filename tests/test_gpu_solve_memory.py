@@ -1,7 +1,7 @@
 """Device memory that a context holds after a one-launch solve, which works on
 a slab of 4 n^2 bytes: at most 256 MB stay (n = 8,000 and below), the slab of a
 larger system goes back, and so does everything with the context (GPU, C ABI).
-The other 96 MB are the margin for the driver's granularity and modules."""
+The other 96 MB are the margin for the allocator's granularity and modules."""
 import numpy as np
 import pytest
 import torch
